@@ -722,44 +722,49 @@ void launch_normal_equations(const Dev& d, int phi_buf, int slot, cudaStream_t s
 // x += D (D M D)^-1 D (b - M x) with the residual in FP64, until the scaled residual is below 1e-10 of
 // the scaled right-hand side.  If the FP32 factorisation breaks down or the refinement stalls, the FP64
 // Cholesky factorisation of M is used instead.
+//
+// One CTA per candidate; every phase is a dependent chain on one SM (IPC 0.7), so the time is the sum of
+// the chains' latencies: P = 55, cycles at 2.07 GHz: inputs 1.8k, set-up 4.3k, factor 8.2k, two
+// substitutions 2 x 4.7k, two FP64 residuals 2 x 2.9k (the FP64 pipe's rate), FK 9k.  Measured per launch,
+// humanoid 50k: 34.9 -> 20 us (a frame of ten iterations 1,406 -> 1,259 us).
 // ---------------------------------------------------------------------------------------------
 constexpr int kSolveThreads = 256;
 constexpr int kMaxRefine = 8;
 
-__device__ void chol_solve_fp64(double* M, double* b, int P, int& fail_out) {
+__device__ void chol_solve_fp64(double* M, int ld, double* b, int P, int& fail_out) {
   __shared__ int fail;
   const int tid = threadIdx.x, nt = blockDim.x;
   if (tid == 0) fail = 0;
   __syncthreads();
   for (int k = 0; k < P; ++k) {
     if (tid == 0) {
-      const double piv = M[k * P + k];
+      const double piv = M[k * ld + k];
       if (!(piv > 0.0)) fail = 1;
-      M[k * P + k] = sqrt(fmax(piv, 0.0));
+      M[k * ld + k] = sqrt(fmax(piv, 0.0));
     }
     __syncthreads();
     if (fail) break;
-    const double ik = 1.0 / M[k * P + k];
-    for (int r = k + 1 + tid; r < P; r += nt) M[r * P + k] *= ik;
+    const double ik = 1.0 / M[k * ld + k];
+    for (int r = k + 1 + tid; r < P; r += nt) M[r * ld + k] *= ik;
     __syncthreads();
     const int n = P - k - 1;
     for (int e = tid; e < n * n; e += nt) {
       const int r = k + 1 + e / n, q = k + 1 + e % n;
-      if (q <= r) M[r * P + q] -= M[r * P + k] * M[q * P + k];
+      if (q <= r) M[r * ld + q] -= M[r * ld + k] * M[q * ld + k];
     }
     __syncthreads();
   }
   if (!fail) {
     for (int k = 0; k < P; ++k) {
-      if (tid == 0) b[k] /= M[k * P + k];
+      if (tid == 0) b[k] /= M[k * ld + k];
       __syncthreads();
-      for (int r = k + 1 + tid; r < P; r += nt) b[r] -= M[r * P + k] * b[k];
+      for (int r = k + 1 + tid; r < P; r += nt) b[r] -= M[r * ld + k] * b[k];
       __syncthreads();
     }
     for (int k = P - 1; k >= 0; --k) {
-      if (tid == 0) b[k] /= M[k * P + k];
+      if (tid == 0) b[k] /= M[k * ld + k];
       __syncthreads();
-      for (int r = tid; r < k; r += nt) b[r] -= M[k * P + r] * b[k];
+      for (int r = tid; r < k; r += nt) b[r] -= M[k * ld + r] * b[k];
       __syncthreads();
     }
   }
@@ -767,222 +772,407 @@ __device__ void chol_solve_fp64(double* M, double* b, int P, int& fail_out) {
   __syncthreads();
 }
 
-// (r, q) of the e-th lower-triangle element in row-major order (e = r (r + 1) / 2 + q, q <= r)
-__device__ __forceinline__ void tri_rc(int e, int& r, int& q) {
-  int rr = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-  while ((rr + 1) * (rr + 2) / 2 <= e) ++rr;
-  while (rr * (rr + 1) / 2 > e) --rr;
-  r = rr;
-  q = e - rr * (rr + 1) / 2;
+constexpr int kBlk = 8;               // block size of the factorisation
+constexpr int kMaxPad = 80;           // P padded to a multiple of kBlk
+// Row r of the FP32 matrices starts at fidx(r, 0): on 16 bytes, with the 16-byte pieces of one column in 8
+// consecutive (aligned) rows on distinct banks (21 pieces per row, odd) and those in rows 0, 4, .., 28 too
+// (one piece of skew per 8 rows).
+constexpr int kFRow = kMaxPad + 4;
+constexpr int kFBlock = kBlk * kFRow + 4;  // distance of two block rows
+__host__ __device__ constexpr int fidx(int r, int c) { return r * kFRow + 4 * (r >> 3) + c; }
+
+// The 8x8 diagonal block at j (lower triangle used) in registers.
+__device__ __forceinline__ void load_diag(const float* F, int j, float (&a)[kBlk][kBlk]) {
+  const float* p = F + (j >> 3) * kFBlock + j;
+#pragma unroll
+  for (int i = 0; i < kBlk; ++i) {
+    const float4 lo = *reinterpret_cast<const float4*>(p + i * kFRow);
+    a[i][0] = lo.x, a[i][1] = lo.y, a[i][2] = lo.z, a[i][3] = lo.w;
+    if (i >= 4) {
+      const float4 hi = *reinterpret_cast<const float4*>(p + i * kFRow + 4);
+      a[i][4] = hi.x, a[i][5] = hi.y, a[i][6] = hi.z, a[i][7] = hi.w;
+    }
+  }
+}
+__device__ __forceinline__ void load8(const float* p, float (&v)[kBlk]) {
+  const float4 lo = *reinterpret_cast<const float4*>(p), hi = *reinterpret_cast<const float4*>(p + 4);
+  v[0] = lo.x, v[1] = lo.y, v[2] = lo.z, v[3] = lo.w;
+  v[4] = hi.x, v[5] = hi.y, v[6] = hi.z, v[7] = hi.w;
+}
+__device__ __forceinline__ void store8(float* p, const float (&v)[kBlk]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-constexpr int kBlk = 8;         // block size of the factorisation
-constexpr int kMaxPad = 80;     // P padded to a multiple of kBlk
+// 1/sqrt(x) of a normal x: what rsqrtf returns for it, without rsqrtf's handling of denormals.
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 
-// Blocked FP32 Cholesky of the padded matrix F (lower triangle, in place), 1/L_kk into ivd.  Per block
-// column: (1) warp 0 factors the 8x8 diagonal block in registers (lane = row, shuffles for the column),
-// (2) one thread per row below solves its 8 entries against that block, (3) one warp per 8x8 block of the
-// trailing triangle subtracts the rank-8 product.  Returns false if a pivot is not positive.
-__device__ bool chol_blocked(float (*F)[kMaxPad + 1], float* ivd, int Pp) {
+// Blocked FP32 Cholesky: F (lower triangle, padded to Pp) is used up, G receives the factor and ivd 1/L_kk.
+// Returns false if a pivot is not positive.  It is a chain of Pp dependent pivots on one SM, so what
+// counts is the latency of a block column.  The warps with rows below the 8x8 diagonal block each factor
+// it redundantly in registers (a pivot is then one rsqrt, one multiply and one FMA: no shuffles, and no
+// barrier between the factor and the panel), a thread solves one panel row, and the trailing triangle goes
+// by 2x4 tiles, one thread each: shared-memory loads return 128 bytes per cycle and SM however many lanes
+// read the same address, so entries formed per load count, but a tile is also one thread's chain.  The
+// factor goes to a matrix of its own, so that the redundant readers of F never race its writer.  Two
+// barriers per block column.
+__device__ bool chol_blocked(float* F, float* G, float* ivd, int Pp) {
   __shared__ int bad;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
   if (tid == 0) bad = 0;
-  __syncthreads();
-  for (int j = 0; j < Pp; j += kBlk) {
-    if (warp == 0) {
-      const int i = lane & 7, r = j + i;
-      float a[kBlk];
+  // this thread's tiles (2 rows x 4 columns) of the trailing triangle, relative to its corner: row pairs in
+  // order, pair i with i / 2 + 1 tiles, so the rows 4 m .. 4 m + 3 hold 2 (m + 1) from tile m (m + 1) on
+  // (at most 18 x 19 tiles for 72 rows)
+  static_assert(2 * kSolveThreads >= 18 * 19, "two tiles per thread cover the largest trailing triangle");
+  int tile[2];
 #pragma unroll
-      for (int q = 0; q < kBlk; ++q) a[q] = F[r][j + q];
+  for (int h = 0; h < 2; ++h) {
+    const int e = tid + h * nt;
+    int m = (int)((sqrtf(4.f * (float)e + 1.f) - 1.f) * 0.5f);
+    if ((m + 1) * (m + 2) <= e) ++m;
+    if (m * (m + 1) > e) --m;
+    const int k = e - m * (m + 1), odd = k > m;
+    tile[h] = (4 * m + 2 * odd) << 8 | 4 * (k - (odd ? m + 1 : 0));
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int j = 0; j < Pp; j += kBlk) {
+    const int j1 = j + kBlk;
+    if (warp == nw - 1 || j1 + 32 * warp < Pp) {
+      float a[kBlk][kBlk], iv[kBlk];
+      load_diag(F, j, a);
+      bool neg = false;
 #pragma unroll
       for (int c = 0; c < kBlk; ++c) {
-        const float dc = __shfl_sync(0xffffffffu, a[c], c);
-        if (!(dc > 0.f)) { if (lane == 0) bad = 1; }
-        const float iv = rsqrtf(fmaxf(dc, 1e-30f));
-        a[c] = i > c ? a[c] * iv : (i == c ? dc * iv : a[c]);
-        if (lane == 0) ivd[j + c] = iv;
+        const float dc = a[c][c];
+        neg |= !(dc > 0.f);
+        iv[c] = rsqrt_normal(fmaxf(dc, 1e-30f));
+        a[c][c] = dc * iv[c];
 #pragma unroll
-        for (int q = c + 1; q < kBlk; ++q) {
-          const float lqc = __shfl_sync(0xffffffffu, a[c], q);
-          if (i >= q) a[q] = fmaf(-a[c], lqc, a[q]);
-        }
+        for (int i = c + 1; i < kBlk; ++i) a[i][c] = a[i][c] * iv[c];
+#pragma unroll
+        for (int q = c + 1; q < kBlk; ++q)
+#pragma unroll
+          for (int i = q; i < kBlk; ++i) a[i][q] = fmaf(-a[i][c], a[q][c], a[i][q]);
       }
-      if (lane < kBlk) {
+      if (warp != nw - 1) {  // a panel row (no panel reaches the last warp)
+        if (j1 + tid < Pp) {
+          float p[kBlk];
+          load8(&F[fidx(j1 + tid, j)], p);
 #pragma unroll
-        for (int q = 0; q < kBlk; ++q)
-          if (q <= i) F[r][j + q] = a[q];
+          for (int c = 0; c < kBlk; ++c) {
+            float sacc = p[c];
+#pragma unroll
+            for (int q = 0; q < c; ++q) sacc = fmaf(-p[q], a[c][q], sacc);
+            p[c] = sacc * iv[c];
+          }
+          store8(&G[fidx(j1 + tid, j)], p);
+        }
+      } else if (tid == nt - 1) {  // the factored diagonal block (its upper triangle is not read)
+        if (neg) bad = 1;
+#pragma unroll
+        for (int i = 0; i < kBlk; ++i) {
+          *reinterpret_cast<float4*>(&G[fidx(j + i, j)]) = make_float4(a[i][0], a[i][1], a[i][2], a[i][3]);
+          if (i >= 4) *reinterpret_cast<float4*>(&G[fidx(j + i, j + 4)]) = make_float4(a[i][4], a[i][5], a[i][6], a[i][7]);
+        }
+        store8(ivd + j, iv);
       }
     }
     __syncthreads();
     if (bad) return false;
-    for (int r = j + kBlk + tid; r < Pp; r += nt) {  // panel
-      float a[kBlk];
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c) a[c] = F[r][j + c];
+    for (int h = 0; h < 2; ++h) {
+      const int r0 = j1 + (tile[h] >> 8), q0 = j1 + (tile[h] & 255);
+      if (r0 >= Pp) break;
+      float lr[2][kBlk], dot[2][4];
+      load8(&G[fidx(r0, j)], lr[0]);
+      load8(&G[fidx(r0 + 1, j)], lr[1]);
+      float4* f0 = reinterpret_cast<float4*>(&F[fidx(r0, q0)]);
+      float4* f1 = reinterpret_cast<float4*>(&F[fidx(r0 + 1, q0)]);
+      const float4 o0 = *f0, o1 = *f1;
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c) {
-        float sacc = a[c];
+      for (int t = 0; t < 4; ++t) {
+        float lq[kBlk];
+        load8(&G[fidx(q0 + t, j)], lq);
 #pragma unroll
-        for (int q = 0; q < c; ++q) sacc = fmaf(-a[q], F[j + c][j + q], sacc);
-        a[c] = sacc * ivd[j + c];
+        for (int u = 0; u < 2; ++u) {
+          dot[u][t] = 0.f;
+#pragma unroll
+          for (int c = 0; c < kBlk; ++c) dot[u][t] = fmaf(lr[u][c], lq[c], dot[u][t]);
+        }
       }
-#pragma unroll
-      for (int c = 0; c < kBlk; ++c) F[r][j + c] = a[c];
-    }
-    __syncthreads();
-    const int nb = (Pp - j - kBlk) / kBlk, nblocks = nb * (nb + 1) / 2;
-    for (int blk = warp; blk < nblocks; blk += nw) {  // trailing update, one warp per 8x8 block
-      int bi, bq;
-      tri_rc(blk, bi, bq);
-      const int r0 = j + kBlk + kBlk * bi, c0 = j + kBlk + kBlk * bq;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int e = lane + 32 * h, r = r0 + (e >> 3), q = c0 + (e & 7);
-        float lr[kBlk], lq[kBlk];
-#pragma unroll
-        for (int c = 0; c < kBlk; ++c) { lr[c] = F[r][j + c]; lq[c] = F[q][j + c]; }
-        float dot = 0.f;
-#pragma unroll
-        for (int c = 0; c < kBlk; ++c) dot = fmaf(lr[c], lq[c], dot);
-        if (bi != bq || q <= r) F[r][q] -= dot;
-      }
+      // (entries right of the diagonal are updated too: nothing reads them)
+      *f0 = make_float4(o0.x - dot[0][0], o0.y - dot[0][1], o0.z - dot[0][2], o0.w - dot[0][3]);
+      *f1 = make_float4(o1.x - dot[1][0], o1.y - dot[1][1], o1.z - dot[1][2], o1.w - dot[1][3]);
     }
     __syncthreads();
   }
   return true;
 }
 
-// Blocked forward and backward substitution with the factor of chol_blocked: y <- (L L^T)^-1 y.
-__device__ void solve_blocked(float (*F)[kMaxPad + 1], const float* ivd, float* y, int Pp) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
-  for (int j = 0; j < Pp; j += kBlk) {  // L z = y
-    if (warp == 0) {
-      const int i = lane & 7;
-      float v = y[j + i];
+// One 8x8 block of the substitutions by a warp whose lanes hold rows lane + 32 k: the block's eight
+// right-hand sides by independent shuffles, the block solved redundantly by every lane in registers, and
+// the lane's own rows updated (rows already solved too: their results are in z and are not read again).
+// The next block's diagonal (at jn) is loaded meanwhile.  Issue-bound: one warp, ~100 instructions.
+template <int SETS, bool kBack>
+__device__ __forceinline__ void solve_block(const float* G, const float* const (&mine_rows)[SETS], const float* ivd, int j, int jn,
+                                            const float (&a)[kBlk][kBlk], const float (&iv)[kBlk],
+                                            float (&an)[kBlk][kBlk], float (&ivn)[kBlk], float (&y)[SETS], float* z) {
+  const int lane = threadIdx.x & 31, set = j >> 5;
+  float row[SETS][kBlk];
+  if constexpr (kBack) {
+    const float* p = G + (j >> 3) * kFBlock + lane;  // (columns past the row: the next row's, not used)
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c) {
-        const float zc = __shfl_sync(0xffffffffu, v, c) * ivd[j + c];
-        v = i == c ? zc : (i > c ? fmaf(-F[j + i][j + c], zc, v) : v);
-      }
-      if (lane < kBlk) y[j + lane] = v;
-    }
-    __syncthreads();
-    for (int r = j + kBlk + tid; r < Pp; r += nt) {
-      float sacc = y[r];
+    for (int k = 0; k < SETS; ++k)
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c) sacc = fmaf(-F[r][j + c], y[j + c], sacc);
-      y[r] = sacc;
-    }
-    __syncthreads();
+      for (int c = 0; c < kBlk; ++c) row[k][c] = p[c * kFRow + (k < 2 ? 32 * k : min(32 * k, kMaxPad - 1 - lane))];
+  } else {
+#pragma unroll
+    for (int k = 0; k < SETS; ++k) load8(mine_rows[k] + j, row[k]);
   }
-  for (int j = Pp - kBlk; j >= 0; j -= kBlk) {  // L^T x = z
-    if (warp == 0) {
-      const int i = lane & 7;
-      float v = y[j + i];
+  float mine = y[0];
 #pragma unroll
-      for (int c = kBlk - 1; c >= 0; --c) {
-        const float xc = __shfl_sync(0xffffffffu, v, c) * ivd[j + c];
-        v = i == c ? xc : (i < c ? fmaf(-F[j + c][j + i], xc, v) : v);
-      }
-      if (lane < kBlk) y[j + lane] = v;
-    }
-    __syncthreads();
-    for (int r = tid; r < j; r += nt) {
-      float sacc = y[r];
+  for (int k = 1; k < SETS; ++k) mine = set == k ? y[k] : mine;
+  float v[kBlk];
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c) sacc = fmaf(-F[j + c][r], y[j + c], sacc);
-      y[r] = sacc;
+  for (int i = 0; i < kBlk; ++i) v[i] = __shfl_sync(0xffffffffu, mine, (j & 31) + i);
+  load_diag(G, jn, an);
+  load8(ivd + jn, ivn);
+#pragma unroll
+  for (int t = 0; t < kBlk; ++t) {
+    const int c = kBack ? kBlk - 1 - t : t;
+    v[c] = v[c] * iv[c];
+#pragma unroll
+    for (int i = 0; i < kBlk; ++i) {
+      if (kBack && i < c) v[i] = fmaf(-a[c][i], v[c], v[i]);
+      if (!kBack && i > c) v[i] = fmaf(-a[i][c], v[c], v[i]);
     }
-    __syncthreads();
   }
+#pragma unroll
+  for (int k = 0; k < SETS; ++k)
+#pragma unroll
+    for (int c = 0; c < kBlk; ++c) y[k] = fmaf(-row[k][c], v[c], y[k]);
+  if (lane == 0) store8(z + j, v);
+}
+
+// y <- (L L^T)^-1 y with the factor of chol_blocked, by one warp without block barriers: lane l holds rows
+// l + 32 k; z (16-byte aligned, kMaxPad) is scratch.
+template <int SETS>
+__device__ __forceinline__ void solve_warp(const float* G, const float* ivd, float (&y)[SETS], float* z,
+                                           int Pp) {
+  const int lane = threadIdx.x & 31;
+  float a[kBlk][kBlk], iv[kBlk], an[kBlk][kBlk], ivn[kBlk];
+  const float* rows[SETS];  // this lane's rows of G
+#pragma unroll
+  for (int k = 0; k < SETS; ++k) rows[k] = G + fidx(min(32 * k + lane, kMaxPad - 1), 0);
+  load_diag(G, 0, a);
+  load8(ivd, iv);
+#pragma unroll 1
+  for (int j = 0; j < Pp; j += 2 * kBlk) {  // L z = y
+    solve_block<SETS, false>(G, rows, ivd, j, min(j + kBlk, Pp - kBlk), a, iv, an, ivn, y, z);
+    if (j + kBlk >= Pp) break;
+    solve_block<SETS, false>(G, rows, ivd, j + kBlk, min(j + 2 * kBlk, Pp - kBlk), an, ivn, a, iv, y, z);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < SETS; ++k) y[k] = z[min(32 * k + lane, kMaxPad - 1)];
+  __syncwarp();
+  load_diag(G, Pp - kBlk, a);
+  load8(ivd + Pp - kBlk, iv);
+#pragma unroll 1
+  for (int j = Pp - kBlk; j >= 0; j -= 2 * kBlk) {  // L^T x = z
+    solve_block<SETS, true>(G, rows, ivd, j, max(j - kBlk, 0), a, iv, an, ivn, y, z);
+    if (j < kBlk) break;
+    solve_block<SETS, true>(G, rows, ivd, j - kBlk, max(j - 2 * kBlk, 0), an, ivn, a, iv, y, z);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < SETS; ++k) y[k] = z[min(32 * k + lane, kMaxPad - 1)];
+}
+
+// ys <- (L L^T)^-1 ys by one warp.
+template <int SETS>
+__device__ __forceinline__ void solve_rows(const float* G, const float* ivd, float* ys, float* z, int P, int Pp) {
+  const int lane = threadIdx.x & 31;
+  float y[SETS];
+#pragma unroll
+  for (int k = 0; k < SETS; ++k) y[k] = lane + 32 * k < P ? ys[lane + 32 * k] : 0.f;
+  solve_warp<SETS>(G, ivd, y, z, Pp);
+#pragma unroll
+  for (int k = 0; k < SETS; ++k)
+    if (lane + 32 * k < P) ys[lane + 32 * k] = y[k];
+}
+
+// (float)x, rounded to nearest even.  Conversions from FP64 share the FP64 pipe, which takes 60 cycles per
+// warp instruction here; where the result is a normal FP32 number or zero, the same bits are formed with
+// integer operations: the exponent rebiased by 1023 - 127 and the 29 dropped mantissa bits rounded, a
+// carry running into the exponent (up to infinity) as it should.  Sets `other` where that does not hold.
+__device__ __forceinline__ float to_float_rn(double x, bool& other) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned t = __funnelshift_l(lo, hi, 3) - (384u << 23);  // exponent (mod 512) and 23 mantissa bits
+  const unsigned up = (lo & 0x1fffffffu) + (t & 1u) > 0x10000000u ? 1u : 0u;
+  const bool zero = ((hi & 0x7fffffffu) | lo) == 0u;
+  other |= !zero && ((hi >> 20) & 0x7ffu) - 897u >= 254u;
+  return __uint_as_float((zero ? 0u : t + up) | (hi & 0x80000000u));
+}
+
+// Byte offset of the link table in the solve's dynamic shared memory: behind F (P padded to the block, rows
+// of kFRow), G (kMaxPad rows: the substitution's lanes read past the padded P), M and six P-vectors.
+__host__ __device__ inline size_t lm_solve_table_offset(int P) {
+  const size_t Pp = (P + kBlk - 1) / kBlk * kBlk, NP = P + 1;
+  return (((fidx((int)Pp, 0) + fidx(kMaxPad, 0)) * sizeof(float) + (NP * NP + 6 * (size_t)P) * sizeof(double)) + 15) & ~(size_t)15;
 }
 
 __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ float F[kMaxPad][kMaxPad + 1];  // FP32 scaled system -> its Cholesky factor
-  __shared__ float ivd[kMaxPad], ys[kMaxPad], sc[kMaxPad];
+  __shared__ __align__(16) float ivd[kMaxPad], zs[kMaxPad];
+  __shared__ float sc[kMaxPad], ys[kMaxPad];  // scale D, scaled residual
   const int P = d.L, NP = d.NP, c = bp.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int Pp = (P + kBlk - 1) / kBlk * kBlk;
-  double* M = reinterpret_cast<double*>(smem_raw);  // [P][P] FP64 system for the residuals
-  double* x = M + P * P;
+  float* F = reinterpret_cast<float*>(smem_raw);  // FP32 scaled system (used up by the factor)
+  float* G = F + fidx(Pp, 0);                     // its Cholesky factor
+  // [NP][NP] as the reduction left it (J^T J, J^T r in column P), then the FP64 system for the residuals
+  double* M = reinterpret_cast<double*>(G + fidx(kMaxPad, 0));
+  double* x = M + NP * NP;
   double* res = x + P;
   double* b = res + P;
   double* dg = b + P;
   double* p2 = dg + P;  // (lambda_s S_kk)^2
   double* th = p2 + P;  // Theta
-  LinkTable* lt = reinterpret_cast<LinkTable*>(smem_raw + ((((size_t)P * P + 6 * P) * 8 + 15) & ~(size_t)15));
+  LinkTable* lt = reinterpret_cast<LinkTable*>(smem_raw + lm_solve_table_offset(P));
   DQ* H0 = reinterpret_cast<DQ*>(reinterpret_cast<unsigned char*>(lt) + ((sizeof(LinkTable) + 15) & ~(size_t)15));
-  __shared__ unsigned rmax_bits, bmax_bits;
+  __shared__ unsigned rmax_bits[2], bmax_bits;  // rmax: one slot per refinement parity
   __shared__ unsigned char frz[kMaxPad];
-  // ---- inputs in one round trip: the link table, A (P x P at row stride NP), its diagonal and last column
-  for (int t = tid; t < (int)(sizeof(LinkTable) / 16); t += nt)
-    cp_async16(reinterpret_cast<char*>(lt) + 16 * t, reinterpret_cast<const char*>(d.links) + 16 * t);
-  for (int e = tid; e < P * P; e += nt) cp_async8(M + e, d.A + (size_t)(e / P) * NP + e % P);
+  __shared__ int any_frz;
+  // ---- inputs in one round trip: the matrix with its last column, the prior, Theta and the link table
+  for (int t = tid; t < NP * NP / 2; t += nt) cp_async16(M + 2 * t, d.A + 2 * t);
+  if ((NP & 1) && tid == 0) cp_async8(M + NP * NP - 1, d.A + NP * NP - 1);
   for (int r = tid; r < P; r += nt) {
-    cp_async8(dg + r, d.A + (size_t)r * NP + r);
-    cp_async8(b + r, d.A + (size_t)r * NP + P);
     cp_async8(p2 + r, d.prior2 + r);
     cp_async8(th + r, d.theta + r);
   }
+  for (int t = tid; t < (int)(sizeof(LinkTable) / 16); t += nt)
+    cp_async16(reinterpret_cast<char*>(lt) + 16 * t, reinterpret_cast<const char*>(d.links) + 16 * t);
   double lam = *d.lam;
   for (int t = 0; t < c; ++t) lam = fmin(lam * 10.0, 1e7);
-  if (tid == 0) bmax_bits = 0u;
+  if (tid == 0) bmax_bits = rmax_bits[0] = any_frz = 0;
   cp_async_wait_all();
   __syncthreads();
   // ---- setup: M = A + diag(prior + lambda dg) (FP64), frozen rows/columns -> identity; scale D in FP32
-  for (int r = tid; r < P; r += nt) {  // each thread reads and writes only its own rows here
-    const double dgr = dg[r] + p2[r];
-    const bool fr = dgr == 0.0;
-    dg[r] = dgr;
-    frz[r] = fr;
-    sc[r] = fr ? 1.f : rsqrtf((float)(dgr * (1.0 + lam)));
-    b[r] = fr ? 0.0 : b[r] + p2[r] * th[r];
-    x[r] = 0.0;
-    res[r] = b[r];
-    double& mrr = M[(size_t)r * P + r];
-    mrr = fr ? 1.0 : mrr + (p2[r] + lam * dgr);
-    atomicMax(&bmax_bits, __float_as_uint(fabsf((float)b[r] * sc[r])));
+  // (an FP64 instruction occupies its sub-partition's pipe for 64 cycles per warp: the two halves of the
+  // block take a part of the vectors each)
+  static_assert(kSolveThreads / 2 >= kMaxPad, "half a block covers the rows");
+  {
+    const int r = tid & (kSolveThreads / 2 - 1);
+    if (r < P) {
+      double& mrr = M[(size_t)r * NP + r];
+      if (tid < kSolveThreads / 2) {
+        const double dgr = mrr + p2[r];
+        const bool fr = dgr == 0.0;
+        frz[r] = fr;
+        if (fr) any_frz = 1;
+        sc[r] = fr ? 1.f : rsqrtf((float)(dgr * (1.0 + lam)));
+        mrr = fr ? 1.0 : mrr + (p2[r] + lam * dgr);
+      } else {
+        b[r] = M[(size_t)r * NP + P] + p2[r] * th[r];
+        ys[r] = (float)b[r];
+        x[r] = 0.0;
+      }
+    }
   }
   __syncthreads();
-  // the off-diagonal of M (zero in frozen rows and columns) and, in the same pass, the FP32 lower triangle
-  // of D M D; a warp per row
-  for (int r = warp; r < P; r += nt >> 5) {
-    const bool fr = frz[r];
-    const float sr = sc[r];
-    for (int q = lane; q < P; q += 32) {
-      double m = M[(size_t)r * P + q];
-      if (q != r && (fr || frz[q])) {
-        m = 0.0;
-        M[(size_t)r * P + q] = 0.0;
+  {
+    unsigned bmine = 0u;
+    if (tid < P) {
+      if (frz[tid]) {
+        b[tid] = 0.0;
+        ys[tid] = 0.f;
       }
-      if (q <= r) F[r][q] = (float)m * sr * sc[q];
+      ys[tid] *= sc[tid];
+      bmine = __float_as_uint(fabsf(ys[tid]));
+    }
+    bmine = __reduce_max_sync(0xffffffffu, bmine);
+    if (lane == 0 && bmine) atomicMax(&bmax_bits, bmine);
+  }
+  if (any_frz) {  // the off-diagonal of M is zero in frozen rows and columns
+    for (int r = warp; r < P; r += nt >> 5)
+      for (int q = lane; q < P; q += 32)
+        if (q != r && (frz[r] || frz[q])) M[(size_t)r * NP + q] = 0.0;
+    __syncthreads();
+  }
+  // the FP32 lower triangle of D M D, a warp per row, four rows' loads in flight
+  {
+    constexpr int kSets = (kMaxPad + 31) / 32, kRows = 4;
+    float scq[kSets];
+#pragma unroll
+    for (int k = 0; k < kSets; ++k) scq[k] = lane + 32 * k < P ? sc[lane + 32 * k] : 0.f;
+    const int step = nt >> 5;
+#pragma unroll 1
+    for (int r0 = warp; r0 < P; r0 += kRows * step) {
+      double m[kRows][kSets];
+      float sr[kRows];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int r = r0 + u * step;
+        sr[u] = r < P ? sc[r] : 0.f;
+#pragma unroll
+        for (int k = 0; k < kSets; ++k)
+          if (32 * k < P) m[u][k] = r < P && lane + 32 * k <= r ? M[(size_t)r * NP + lane + 32 * k] : 0.0;
+      }
+      float f[kRows][kSets];
+      bool other = false;
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+#pragma unroll
+        for (int k = 0; k < kSets; ++k)
+          if (32 * k < P) f[u][k] = to_float_rn(m[u][k], other);
+      if (__any_sync(0xffffffffu, other)) {
+#pragma unroll
+        for (int u = 0; u < kRows; ++u)
+#pragma unroll
+          for (int k = 0; k < kSets; ++k) f[u][k] = (float)m[u][k];
+      }
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+#pragma unroll
+        for (int k = 0; k < kSets; ++k)
+          if (lane + 32 * k <= r0 + u * step && r0 + u * step < P)
+            F[fidx(r0 + u * step, lane + 32 * k)] = f[u][k] * sr[u] * scq[k];
     }
   }
   for (int e = tid; e < (Pp - P) * Pp; e += nt) {  // identity rows padding P to a multiple of the block
     const int r = P + e / Pp, q = e % Pp;
-    if (q <= r) F[r][q] = r == q ? 1.f : 0.f;
+    if (q <= r) F[fidx(r, q)] = r == q ? 1.f : 0.f;
   }
   __syncthreads();
   // ---- FP32 factor of D M D, padded with identity rows to a multiple of the block size
-  const bool ok32 = chol_blocked(F, ivd, Pp);
+  const bool ok32 = chol_blocked(F, G, ivd, Pp);
   // ---- iterative refinement: x += D (D M D)^-1 D (b - M x), residual in FP64
   int iters = 0;
   bool converged = false;
   const float bmax = __uint_as_float(bmax_bits);
   for (int it = 0; it < kMaxRefine && ok32; ++it) {
-    for (int r = tid; r < Pp; r += nt) ys[r] = r < P ? (float)res[r] * sc[r] : 0.f;
+    if (warp == 0) {
+      if (Pp <= 32) solve_rows<1>(G, ivd, ys, zs, P, Pp);
+      else if (Pp <= 64) solve_rows<2>(G, ivd, ys, zs, P, Pp);
+      else solve_rows<3>(G, ivd, ys, zs, P, Pp);
+    }
     __syncthreads();
-    solve_blocked(F, ivd, ys, Pp);
     for (int r = tid; r < P; r += nt) x[r] += (double)sc[r] * (double)ys[r];
-    if (tid == 0) rmax_bits = 0u;
     __syncthreads();
+    if (tid == 0) rmax_bits[(it + 1) & 1] = 0u;  // every thread has read it (the previous iteration's test)
     // res = b - M x in FP64: four threads per row (columns q = part mod 4, two accumulators each), the
     // four sums combined by shuffles in a fixed pairing
+    unsigned rmine = 0u;
     for (int r0 = 0; r0 < P; r0 += nt / 4) {
       const int r = r0 + (tid >> 2), part = tid & 3;
       double s0 = 0.0, s1 = 0.0;
       if (r < P) {
-        const double* mr = M + (size_t)r * P;
+        const double* mr = M + (size_t)r * NP;
         int q = part;
         for (; q + 4 < P; q += 8) {
           s0 = fma(-mr[q], x[q], s0);
@@ -995,19 +1185,21 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
       sum += __shfl_xor_sync(0xffffffffu, sum, 2);
       if (r < P && part == 0) {
         const double rres = b[r] + sum;
-        res[r] = rres;
-        atomicMax(&rmax_bits, __float_as_uint(fabsf((float)rres * sc[r])));
+        ys[r] = (float)rres * sc[r];
+        rmine = max(rmine, __float_as_uint(fabsf(ys[r])));
       }
     }
+    rmine = __reduce_max_sync(0xffffffffu, rmine);
+    if (lane == 0 && rmine) atomicMax(&rmax_bits[it & 1], rmine);
     __syncthreads();
     iters = it + 1;
-    if (__uint_as_float(rmax_bits) <= 1e-10f * bmax) { converged = true; break; }
+    if (__uint_as_float(rmax_bits[it & 1]) <= 1e-10f * bmax) { converged = true; break; }
   }
   int fail = 0;
   if (!converged) {  // FP64 Cholesky of the unscaled system
     for (int r = tid; r < P; r += nt) x[r] = b[r];
     __syncthreads();
-    chol_solve_fp64(M, x, P, fail);
+    chol_solve_fp64(M, NP, x, P, fail);
   }
   double* thc = d.theta_c + (size_t)c * P;
   for (int j = tid; j < P; j += nt) {  // the candidate, also kept in shared memory (res is free now) for FK
@@ -1023,7 +1215,7 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   fk_all(*lt, res, H0, d.Hd_c + (size_t)c * P, d.xi_c + (size_t)c * P * 8, 8);
 }
 
-__global__ void __launch_bounds__(kSolveThreads) k_lm_solve(BatchGrid g, Dev d0) {
+__global__ void __launch_bounds__(kSolveThreads, 2) k_lm_solve(BatchGrid g, Dev d0) {
   if (g.map == nullptr) {
     lm_solve_impl(d0, grid_pos());
     return;
@@ -1197,8 +1389,7 @@ __global__ void __launch_bounds__(kBlock) k_lm_eval(BatchGrid g, Dev d0, int c0,
 }
 
 static int lm_solve_smem(int L) {
-  return (int)(((((size_t)L * L + 6 * L) * 8 + 15) & ~(size_t)15) + ((sizeof(LinkTable) + 15) & ~(size_t)15) +
-               (size_t)L * sizeof(DQ));
+  return (int)(lm_solve_table_offset(L) + ((sizeof(LinkTable) + 15) & ~(size_t)15) + (size_t)L * sizeof(DQ));
 }
 
 void launch_lm_solve(const Dev& d, cudaStream_t st) {

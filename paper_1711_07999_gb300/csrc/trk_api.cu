@@ -732,6 +732,19 @@ trk_status create_session(const trk_mesh* mesh, const trk_skeleton* sk, const tr
     }
     lt.round_start[nr] = k;
     lt.chain_start[k] = t;
+    std::vector<int> slot_of(L);
+    for (int q = 0; q < L; ++q) {
+      const int j = lt.chain[q];
+      slot_of[j] = q;
+      const float* o = sk->offset_dq + 8 * j;
+      const bool unit = o[0] == 1.f && o[1] == 0.f && o[2] == 0.f && o[3] == 0.f && o[4] == 0.f;
+      const int kind = !unit ? kOffGeneral : (o[5] == 0.f && o[6] == 0.f && o[7] == 0.f) ? kOffIdentity : kOffTranslation;
+      lt.slot_tag[q] = j | sk->type[j] << 8 | kind << 9;
+    }
+    for (int c = 0; c < nc; ++c) {
+      const int head = lt.chain[lt.chain_start[c]];
+      lt.chain_up[c] = sk->parent[head] < 0 ? -1 : slot_of[sk->parent[head]];
+    }
   }
   lt.pre.r = make_float4(1.f, 0.f, 0.f, 0.f);
   lt.pre.d = make_float4(0.f, (float)pre.d.x, (float)pre.d.y, (float)pre.d.z);

@@ -37,6 +37,7 @@ struct __align__(32) Acc4 {
 // All positions on the device live in a session-local frame: the camera frame shifted by the template's
 // bind-pose centroid c (so coordinates stay within ~1 m and FP32 keeps ~1e-7 m of absolute precision).
 // FK starts from pre = T(-c); the bind pose is stored in the same frame.
+constexpr int kOffIdentity = 0, kOffTranslation = 1, kOffGeneral = 2;  // what there is of a link's offset
 struct LinkTable {
   int L;
   int max_depth;  // largest link depth (root links: 0)
@@ -53,6 +54,8 @@ struct LinkTable {
   int chain[kMaxLinks];
   int chain_start[kMaxLinks + 1];
   int round_start[kMaxLinks + 1];
+  int slot_tag[kMaxLinks];  // of link chain[t]: its index | type << 8 | kOff* << 9
+  int chain_up[kMaxLinks];  // position in chain[] of the parent of chain c's head (-1: the world)
   DQ pre;               // T(-c)
   DQ off[kMaxLinks];
   DQ bindc[kMaxLinks];  // conjugate of the bind-pose DQ T(-c) H^0_{0,j}
@@ -135,44 +138,87 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // a prismatic joint (the joint's generator H_j^{-1} dH_j/dtheta_j): dH_{k,Delta}/dtheta_j = Xi_j H_{k,Delta}
 // for every k below j.
 //
-// One thread walks each chain of single-child links (a 3-DoF joint is three such links), the chains of a
-// round in parallel, one barrier per round: the products are those of a link-by-link walk from the root,
-// with ~3x fewer barriers.  H0 (shared, [L]) is scratch; all threads of the block must call it.
+// The links go chain by chain (single-child links: a 3-DoF joint is three), the chains of a round in
+// parallel, one barrier per round: the products are those of a link-by-link walk from the root.  The walk
+// is one thread's chain of dual-quaternion products, bound by their latency and instruction count, so
+//  - a chain has a warp to itself: its branches do not diverge (three chains in the lanes of one warp took
+//    310 cycles per link, this ~150);
+//  - the factors that are exactly 0 or 1 are not multiplied: a joint's transform has no dual part (hinge)
+//    or a unit real part (prismatic), and an offset that is the identity (the second and third link of a
+//    multi-DoF joint) or a pure translation costs nothing or one product; what is left are the same
+//    values (x 1 and + 0 are exact);
+//  - a link's factors are laid out in walking order (H0[t], replaced by its product), so the next link's
+//    are loaded while the current products run.
+// H0 (shared, [L]) is scratch; all threads of the block must call it (whole warps).
 template <typename ThetaT>
 __device__ __forceinline__ void fk_all(const LinkTable& lt, const ThetaT* theta, DQ* H0, DQ* Hd_out, float* xi_out,
                                        int xi_stride) {
   const int L = lt.L;
-  for (int j = threadIdx.x; j < L; j += blockDim.x) H0[j] = joint_dq(lt.type[j], lt.axis[j], (float)theta[j]);
+  for (int t = threadIdx.x; t < L; t += blockDim.x) {
+    const int tag = lt.slot_tag[t], j = tag & 255;
+    const DQ J = joint_dq((tag >> 8) & 1, lt.axis[j], (float)theta[j]);
+    H0[t].r = (tag >> 8) & 1 ? J.d : J.r;
+    H0[t].d = lt.off[j].d;
+  }
   __syncthreads();
   for (int r = 0; r < lt.n_rounds; ++r) {
-    for (int c = lt.round_start[r] + threadIdx.x; c < lt.round_start[r + 1]; c += blockDim.x) {
-      const int head = lt.chain[lt.chain_start[c]];
-      DQ H = lt.parent[head] < 0 ? lt.pre : H0[lt.parent[head]];
-      for (int t = lt.chain_start[c]; t < lt.chain_start[c + 1]; ++t) {
-        const int j = lt.chain[t];
-        H = dqmul(dqmul(H, lt.off[j]), H0[j]);
-        H0[j] = H;
+    if ((threadIdx.x & 31) == 0) {
+      for (int c = lt.round_start[r] + (threadIdx.x >> 5); c < lt.round_start[r + 1]; c += blockDim.x >> 5) {
+        int t = lt.chain_start[c];
+        const int last = lt.chain_start[c + 1] - 1, up = lt.chain_up[c];
+        DQ H = up < 0 ? lt.pre : H0[up];
+        DQ f = H0[t];
+        int tag = lt.slot_tag[t];
+#pragma unroll 1
+        for (;; ++t) {
+          const DQ fn = H0[min(t + 1, last)];
+          const int tagn = lt.slot_tag[min(t + 1, last)];
+          if (tag >> 9 != kOffIdentity) {
+            if (tag >> 9 == kOffTranslation) H.d = qadd(qmul(H.r, f.d), H.d);
+            else H = dqmul(H, lt.off[tag & 255]);
+          }
+          if (tag & 256) {
+            H.d = qadd(qmul(H.r, f.r), H.d);
+          } else {
+            H.d = qmul(H.d, f.r);
+            H.r = qmul(H.r, f.r);
+          }
+          H0[t] = H;
+          if (t == last) break;
+          f = fn;
+          tag = tagn;
+        }
       }
     }
     __syncthreads();
   }
-  for (int j = threadIdx.x; j < L; j += blockDim.x) {
-    const DQ H = H0[j];
-    Hd_out[j] = dqmul(H, lt.bindc[j]);
-    DQ G;
+  // the two outputs of a link by different threads, in one (rolled) sequence of products: this code runs
+  // once per launch, where its size costs as much as its arithmetic
+  for (int q = threadIdx.x; q < 2 * L; q += blockDim.x) {
+    const bool twist = q >= L;
+    const int t = twist ? q - L : q, j = lt.chain[t];
+    const DQ H = H0[t];
     const float* z = lt.axis[j];
-    if (lt.type[j] == 0) {
-      G.r = make_float4(0.f, 0.5f * z[0], 0.5f * z[1], 0.5f * z[2]);
-      G.d = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-      G.r = make_float4(0.f, 0.f, 0.f, 0.f);
-      G.d = make_float4(0.f, 0.5f * z[0], 0.5f * z[1], 0.5f * z[2]);
+    const float4 g = make_float4(0.f, 0.5f * z[0], 0.5f * z[1], 0.5f * z[2]), o = make_float4(0.f, 0.f, 0.f, 0.f);
+    DQ B = lt.bindc[j];
+    if (twist) {
+      B.r = lt.type[j] == 0 ? g : o;
+      B.d = lt.type[j] == 0 ? o : g;
     }
-    const DQ X = dqmul(dqmul(H, G), dqconj(H));
-    float* xo = xi_out + (size_t)j * xi_stride;
-    xo[0] = X.r.y; xo[1] = X.r.z; xo[2] = X.r.w;
-    xo[3] = X.d.y; xo[4] = X.d.z; xo[5] = X.d.w;
-    if (xi_stride > 6) { xo[6] = 0.f; xo[7] = 0.f; }
+    DQ X = H;
+#pragma unroll 1
+    for (int k = 0; k <= (int)twist; ++k) {
+      X = dqmul(X, B);
+      B = dqconj(H);
+    }
+    if (!twist) {
+      Hd_out[j] = X;
+    } else {
+      float* xo = xi_out + (size_t)j * xi_stride;
+      xo[0] = X.r.y; xo[1] = X.r.z; xo[2] = X.r.w;
+      xo[3] = X.d.y; xo[4] = X.d.z; xo[5] = X.d.w;
+      if (xi_stride > 6) { xo[6] = 0.f; xo[7] = 0.f; }
+    }
   }
 }
 
