@@ -584,6 +584,10 @@ __global__ void __launch_bounds__(kBlock) k_resid_jtj_tc(BatchGrid g, Dev d0, in
 // u |S| + (n u)^2 sum |x| in FP32 unit roundoff u, i.e. as if added in twice the precision).  The FP64
 // pipe issues a small fraction of the FP32 rate on this GPU, so it is left to warp 0, which adds the 32
 // warp sums (hi + lo) in FP64 in warp order.
+//
+// What bounds it is latency: one round trip for the partials, then the FP64 chain over the warps' sums
+// (64 cycles an addition).  Humanoid 50k / 640x480 (196 partials of 1,596 entries): 14.6 -> 6.6 us; the
+// prior term of E was a chain of 55 x 3 FP64 operations in one thread, the last partials one load at a time.
 constexpr int kReduceThreads = 1024;
 
 __device__ __forceinline__ void sum2_add(float& hi, float& lo, float x) {
@@ -594,52 +598,79 @@ __device__ __forceinline__ void sum2_add(float& hi, float& lo, float x) {
   lo += e;
 }
 
+// (double)x of a normal x or zero, with integer operations: conversions to FP64 take 60 cycles of the FP64
+// pipe per warp.  Sets `other` where x is neither.
+__device__ __forceinline__ double widen(float x, bool& other) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+  other |= a != 0u && a - 0x00800000u >= 0x7f000000u;
+  const unsigned hi = (u & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(a << 29));
+}
+
+constexpr int kReduceBatch = 8;  // partials a warp has in flight
+
 __device__ __forceinline__ void reduce_jtj_impl(const Dev& d, BlockPos bp, int slot) {
   __shared__ double sm[kReduceThreads / 32][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int NP = d.NP, n2 = NP * NP, nu = NP * (NP + 1) / 2;
-  // lane -> the u-th entry of the upper triangle, row-major: (r, c), r <= c, at e = r NP + c
+  // lane -> the u-th entry of the upper triangle, row-major: (r, c), r <= c, at e = r NP + c; counted from
+  // the end, row NP - 1 - m holds m + 1 entries
   const int u = bp.x * 32 + lane;
   int r = 0, c = 0;
   if (u < nu) {
-    int rest = u;
-    while (rest >= NP - r) rest -= NP - r++;
-    c = r + rest;
+    const int v = nu - 1 - u;
+    int m = (int)((sqrtf(8.f * (float)v + 1.f) - 1.f) * 0.5f);
+    if ((m + 1) * (m + 2) / 2 <= v) ++m;
+    if (m * (m + 1) / 2 > v) --m;
+    r = NP - 1 - m;
+    c = NP - 1 - (v - m * (m + 1) / 2);
   }
   const int e = r * NP + c;
-  // warp w < S takes blocks w, w + S, ... (four loads in flight together, each partial loaded with its row
-  // count rather than after it); blocks that added no rows wrote no partial and count as zero.  S depends
-  // on the session alone, so its sums have the same order in any launch.
+  // warp w < S takes blocks w, w + S, ... (up to kReduceBatch loads in flight together, each partial loaded
+  // with its row count rather than after it); blocks that added no rows wrote no partial and count as
+  // zero.  S depends on the session alone, so its sums have the same order in any launch.
   const int nb = d.nblk_rows;
   const int S = reduce_warps(nb);
   float hi = 0.f, lo = 0.f;
   if (u < nu && w < S) {
-    int b = w;
-    for (; b + 3 * S < nb; b += 4 * S) {
-      const int r0 = d.jtj_rows[b], r1 = d.jtj_rows[b + S], r2 = d.jtj_rows[b + 2 * S], r3 = d.jtj_rows[b + 3 * S];
-      const float q0 = d.partial[(size_t)b * n2 + e], q1 = d.partial[(size_t)(b + S) * n2 + e];
-      const float q2 = d.partial[(size_t)(b + 2 * S) * n2 + e], q3 = d.partial[(size_t)(b + 3 * S) * n2 + e];
-      sum2_add(hi, lo, r0 > 0 ? q0 : 0.f);
-      sum2_add(hi, lo, r1 > 0 ? q1 : 0.f);
-      sum2_add(hi, lo, r2 > 0 ? q2 : 0.f);
-      sum2_add(hi, lo, r3 > 0 ? q3 : 0.f);
-    }
-    for (; b < nb; b += S) {
-      const int rows = d.jtj_rows[b];
-      const float q = d.partial[(size_t)b * n2 + e];
-      if (rows > 0) sum2_add(hi, lo, q);
+    for (int b0 = w; b0 < nb; b0 += kReduceBatch * S) {
+      int rows[kReduceBatch];
+      float q[kReduceBatch];
+#pragma unroll
+      for (int k = 0; k < kReduceBatch; ++k) {
+        const int b = b0 + k * S;
+        rows[k] = b < nb ? d.jtj_rows[b] : 0;
+        q[k] = b < nb ? d.partial[(size_t)b * n2 + e] : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < kReduceBatch; ++k) sum2_add(hi, lo, rows[k] > 0 ? q[k] : 0.f);
     }
   }
-  sm[w][lane] = (double)hi + (double)lo;
+  // E's prior term by the block that holds the last entry (NP - 1, NP - 1), a warp beside the sums
+  const bool has_e = bp.x == (nu - 1) / 32;
+  __shared__ double prior;
+  if (has_e && w == (blockDim.x >> 5) - 1) {
+    double p = 0.0;
+    for (int k = lane; k < d.L; k += 32) p += d.prior2[k] * d.theta[k] * d.theta[k];
+    for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+    if (lane == 0) prior = p;
+  }
+  bool other = false;
+  double dh = widen(hi, other), dl = widen(lo, other);
+  if (__any_sync(0xffffffffu, other)) {
+    dh = (double)hi;
+    dl = (double)lo;
+  }
+  sm[w][lane] = dh + dl;
   __syncthreads();
   if (w != 0 || u >= nu) return;
   double t = 0.0;
+#pragma unroll 8
   for (int k = 0; k < S; ++k) t += sm[k][lane];
   d.A[e] = t;
   d.A[c * NP + r] = t;  // A is symmetric: the lower triangle mirrors the upper
   if (e == n2 - 1) {
-    double E = t;
-    for (int k = 0; k < d.L; ++k) E += d.prior2[k] * d.theta[k] * d.theta[k];
+    const double E = t + prior;
     if (slot >= 0) d.energy[slot] = E;
     d.lm_trials[6] = E;
   }
@@ -1060,6 +1091,10 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   double lam = *d.lam;
   for (int t = 0; t < c; ++t) lam = fmin(lam * 10.0, 1e7);
   if (tid == 0) bmax_bits = rmax_bits[0] = any_frz = 0;
+  if (tid == nt - 1) {  // lambda after the step if this candidate is taken; if none is, after the last one
+    d.lam_next[c] = fmax(lam / 10.0, 1e-7);
+    if (c == kCandidates - 1) d.lam_next[kCandidates] = fmin(lam * 10.0, 1e7);
+  }
   cp_async_wait_all();
   __syncthreads();
   // ---- setup: M = A + diag(prior + lambda dg) (FP64), frozen rows/columns -> identity; scale D in FP32
@@ -1233,9 +1268,15 @@ __global__ void __launch_bounds__(kSolveThreads, 2) k_lm_solve(BatchGrid g, Dev 
 // their energies and marks the step pending (lm_trials[7] = -2), and the second pass scores candidates
 // 2-5 and decides over all six.  The decision sequence and every energy are those of scoring all six at
 // once (each candidate's sum has the same blocks in the same order).  Candidates not scored report +inf.
+//
+// A chain of round trips: row count, records, ticket, block energies, decision, tables.  FP64 additions
+// (64 cycles each and warp) are kept out of it where they can be: only the scored candidates are added, a
+// warp per candidate, and the next lambdas come from the solve.  Humanoid 50k, first pass: 12.6 -> 10.3 us
+// alone, 39 -> 31 us for 16 sessions.
 constexpr double kPending = -2.0;
 
-__device__ __forceinline__ void lm_eval_impl(const Dev& d, BlockPos bp, int c0, int c1) {
+template <int c0, int c1>  // the candidates it scores
+__device__ __forceinline__ void lm_eval_impl(const Dev& d, BlockPos bp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   DQ* sH = reinterpret_cast<DQ*>(smem_raw);  // [kCandidates][L]
   __shared__ int sok[kCandidates];
@@ -1289,76 +1330,54 @@ __device__ __forceinline__ void lm_eval_impl(const Dev& d, BlockPos bp, int c0, 
     for (int o = 16; o > 0; o >>= 1) e[c] += __shfl_xor_sync(0xffffffffu, e[c], o);
   if (lane == 0) {
 #pragma unroll
-    for (int c = 0; c < kCandidates; ++c) swarp[w][c] = e[c];
+    for (int c = 0; c < kCandidates; ++c)
+      if (c >= c0 && c < c1) swarp[w][c] = e[c];
   }
   __syncthreads();
-  if (tid >= c0 && tid < c1) {
-    double s = 0.0;
-    for (int k = 0; k < kBlock / 32; ++k) s += swarp[k][tid];
-    d.epart[(size_t)bp.x * 8 + tid] = s;
+  // the block's energies, then its ticket: one warp writes, fences and takes it
+  if (w == 0) {
+    if (lane >= c0 && lane < c1) {
+      double s = 0.0;
+#pragma unroll
+      for (int k = 0; k < kBlock / 32; ++k) s += swarp[k][lane];
+      d.epart[(size_t)bp.x * 8 + lane] = s;
+      __threadfence();
+    }
+    __syncwarp();
+    if (lane == 0) last = atomicAdd(&d.counter[0], 1u) == (unsigned)bp.gx - 1;
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) last = atomicAdd(&d.counter[0], 1u) == (unsigned)bp.gx - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();
-  // the session's last block: sum of the block energies (strided over the threads, then a shuffle tree
-  // and the 8 warp sums in order) plus each candidate's prior term (warp c, lanes over the links)
-  __shared__ double Ec[kCandidates], pri[kCandidates];
-  {
-    double s6[kCandidates] = {0, 0, 0, 0, 0, 0};
-    for (int b = tid; b < bp.gx; b += kBlock) {
-#pragma unroll
-      for (int c = 0; c < kCandidates; ++c)
-        if (c >= c0 && c < c1) s6[c] += __ldcg(d.epart + (size_t)b * 8 + c);
-    }
-#pragma unroll
-    for (int c = 0; c < kCandidates; ++c)
-      for (int o = 16; o > 0; o >>= 1) s6[c] += __shfl_xor_sync(0xffffffffu, s6[c], o);
-    __syncthreads();  // swarp is reused
-    if (lane == 0) {
-#pragma unroll
-      for (int c = 0; c < kCandidates; ++c) swarp[w][c] = s6[c];
-    }
+  // the session's last block: warp c adds candidate c's block energies and prior terms (strided over the
+  // lanes, then a shuffle tree)
+  __shared__ double Ec[kCandidates];
+  const double inf = __longlong_as_double(0x7ff0000000000000ll);
+  if (w < kCandidates) {
+    double v = 0.0;
     if (w >= c0 && w < c1) {
       const double* thc = d.theta_c + (size_t)w * L;
-      double p = 0.0;
-      for (int k = lane; k < L; k += 32) p += d.prior2[k] * thc[k] * thc[k];
-      for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-      if (lane == 0) pri[w] = p;
-    }
-  }
-  __syncthreads();
-  const double inf = __longlong_as_double(0x7ff0000000000000ll);
-  if (tid < kCandidates) {
-    if (tid >= c0 && tid < c1) {
-      double s = 0.0;
-      for (int k = 0; k < kBlock / 32; ++k) s += swarp[k][tid];
-      Ec[tid] = sok[tid] ? s + pri[tid] : inf;
+#pragma unroll 4
+      for (int k = lane; k < L; k += 32) v += d.prior2[k] * thc[k] * thc[k];
+#pragma unroll 8
+      for (int b = lane; b < bp.gx; b += 32) v += __ldcg(d.epart + (size_t)b * 8 + w);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (!sok[w]) v = inf;
     } else {
-      Ec[tid] = tid < c0 ? d.lm_trials[tid] : inf;  // the first pass's energies; later ones unscored
+      v = w < c0 ? d.lm_trials[w] : inf;  // the first pass's energies; later ones unscored
     }
+    if (lane == 0) Ec[w] = v;
   }
   __syncthreads();
   __shared__ int acc_c;
   if (tid == 0) {
     const double E = d.lm_trials[6];
-    double lam = *d.lam;
     int a = -1;
-    for (int c = 0; c < c1; ++c) {
-      d.lm_trials[c] = Ec[c];
-      if (a < 0 && sok[c] && Ec[c] <= E) a = c;
-    }
-    for (int c = c1; c < kCandidates; ++c) d.lm_trials[c] = inf;
+#pragma unroll
+    for (int c = kCandidates - 1; c >= 0; --c)
+      if (c < c1 && sok[c] && Ec[c] <= E) a = c;
     if (a >= 0 || c1 == kCandidates) {
-      if (a >= 0) {
-        for (int t = 0; t < a; ++t) lam = fmin(lam * 10.0, 1e7);
-        lam = fmax(lam / 10.0, 1e-7);
-      } else {
-        for (int t = 0; t < kCandidates; ++t) lam = fmin(lam * 10.0, 1e7);
-      }
-      *d.lam = lam;
+      *d.lam = d.lam_next[a >= 0 ? a : kCandidates];
       d.lm_trials[7] = (double)a;
     } else {
       d.lm_trials[7] = kPending;
@@ -1366,26 +1385,30 @@ __device__ __forceinline__ void lm_eval_impl(const Dev& d, BlockPos bp, int c0, 
     acc_c = a;
     d.counter[0] = 0;
   }
+  if (tid < kCandidates) d.lm_trials[tid] = tid < c1 ? Ec[tid] : inf;
   __syncthreads();
   const int a = acc_c;
-  if (a >= 0) {
-    for (int j = tid; j < L; j += kBlock) {
-      d.theta[j] = d.theta_c[(size_t)a * L + j];
-      d.Hd[j] = d.Hd_c[(size_t)a * L + j];
-      for (int q = 0; q < 8; ++q) d.xi[8 * j + q] = d.xi_c[((size_t)a * L + j) * 8 + q];
+  if (a >= 0) {  // the accepted candidate's Theta and tables, in 16-byte pieces (a piece per thread)
+    const float4* H = reinterpret_cast<const float4*>(d.Hd_c + (size_t)a * L);
+    const float4* X = reinterpret_cast<const float4*>(d.xi_c + (size_t)a * L * 8);
+    for (int t = tid; t < 4 * L; t += kBlock) {
+      if (t < 2 * L) reinterpret_cast<float4*>(d.Hd)[t] = H[t];
+      else reinterpret_cast<float4*>(d.xi)[t - 2 * L] = X[t - 2 * L];
     }
+    for (int j = tid; j < L; j += kBlock) d.theta[j] = d.theta_c[(size_t)a * L + j];
   }
 }
 
 constexpr int kFirstPass = 2;  // candidates scored by the first pass
 
-__global__ void __launch_bounds__(kBlock) k_lm_eval(BatchGrid g, Dev d0, int c0, int c1) {
+template <int c0, int c1>
+__global__ void __launch_bounds__(kBlock) k_lm_eval(BatchGrid g, Dev d0) {
   if (g.map == nullptr) {
-    lm_eval_impl(d0, grid_pos(), c0, c1);
+    lm_eval_impl<c0, c1>(d0, grid_pos());
     return;
   }
   __shared__ Dev sd;
-  lm_eval_impl(sd, batch_block(g, sd), c0, c1);
+  lm_eval_impl<c0, c1>(sd, batch_block(g, sd));
 }
 
 static int lm_solve_smem(int L) {
@@ -1398,8 +1421,8 @@ void launch_lm_solve(const Dev& d, cudaStream_t st) {
 
 void launch_lm_eval(const Dev& d, int /*phi_buf: the rows' records already hold x0 + phi*/, cudaStream_t st) {
   const size_t sm = kCandidates * d.L * sizeof(DQ);
-  k_lm_eval<<<d.nblk_rows, kBlock, sm, st>>>(kSingle, d, 0, kFirstPass);
-  k_lm_eval<<<d.nblk_rows, kBlock, sm, st>>>(kSingle, d, kFirstPass, kCandidates);
+  k_lm_eval<0, kFirstPass><<<d.nblk_rows, kBlock, sm, st>>>(kSingle, d);
+  k_lm_eval<kFirstPass, kCandidates><<<d.nblk_rows, kBlock, sm, st>>>(kSingle, d);
 }
 
 void launch_lm(const Dev& d, int phi_buf, cudaStream_t st) {
@@ -1856,8 +1879,8 @@ void launch_lm_b(const BatchGrid& glm, int nlm, const BatchGrid& gv, int nv, int
   if (nlm > 0) k_lm_solve<<<nlm, kSolveThreads, lm_solve_smem(max_links), st>>>(glm, Dev{});
   if (nv > 0) {
     const size_t sm = kCandidates * max_links * sizeof(DQ);
-    k_lm_eval<<<nv, kBlock, sm, st>>>(gv, Dev{}, 0, kFirstPass);
-    k_lm_eval<<<nv, kBlock, sm, st>>>(gv, Dev{}, kFirstPass, kCandidates);
+    k_lm_eval<0, kFirstPass><<<nv, kBlock, sm, st>>>(gv, Dev{});
+    k_lm_eval<kFirstPass, kCandidates><<<nv, kBlock, sm, st>>>(gv, Dev{});
   }
 }
 

@@ -531,7 +531,7 @@ void carve_all(trk_session* s) {
   carve(s, &d.energy, std::max(1, prm.pose_iters + prm.shape_iters));
   carve(s, &d.Hd, L); carve(s, &d.xi, (size_t)8 * L);
   carve(s, &d.theta_c, (size_t)kCandidates * L); carve(s, &d.Hd_c, (size_t)kCandidates * L);
-  carve(s, &d.xi_c, (size_t)kCandidates * L * 8); carve(s, &d.lm_trials, 8);
+  carve(s, &d.xi_c, (size_t)kCandidates * L * 8); carve(s, &d.lm_trials, 8); carve(s, &d.lam_next, kCandidates + 1);
   carve(s, &d.lm_ok, 2 * kCandidates);
   carve(s, &d.v, V); carve(s, &d.n, V); carve(s, &d.fn, F); carve(s, &d.rec, V);
   carve(s, &d.head, npx); carve(s, &d.zbuf, npx); carve(s, &d.corr, npx);

@@ -345,6 +345,7 @@ struct Dev {
   DQ* Hd_c;         // [kCandidates][L]
   float* xi_c;      // [kCandidates][L][8]
   double* lm_trials;  // [8]
+  double* lam_next;   // [kCandidates + 1] lambda after the step that takes candidate c; after none
   int* lm_ok;         // [kCandidates] ok flags, then [kCandidates] solver diagnostics
   // per-iteration buffers
   float4* v;
