@@ -1,9 +1,9 @@
 // kernels_jtj.cu -- the contraction [J r]^T [J r] of materialised FP32 rows (Eqs. JTJ, JTr), as a
 // standalone operation on caller device buffers.
 //
-// Each CTA takes a contiguous range of rows, stages them 64 at a time in shared memory and accumulates
-// its (16T) x (16T) product in registers (16 x 16 threads, a T x T tile each); the per-CTA partials are
-// then added in CTA order in FP64 (deterministic for a given grid).
+// Each CTA takes a contiguous range of rows and adds them in order: every output entry is one chain of
+// multiply-adds per CTA, and the per-CTA partials are then added in CTA order in FP64 (deterministic for a
+// given grid).
 #include <algorithm>
 #include <cstdio>
 #include <mutex>
@@ -14,90 +14,234 @@
 
 namespace trk {
 
-constexpr int kJBlock = 256;
-constexpr int kJStage = 64;
+constexpr int kJBlock = 256;      // rows that make a CTA worth having (the grid's rule)
+constexpr int kJStage = 16;       // rows per pipeline stage
+constexpr int kJStages = 4;
+constexpr int kJLoaders = 64;     // threads that only load
 constexpr int kJMaxBlocks = 296;
 
-template <int T>
-__global__ void __launch_bounds__(kJBlock) k_jtj_rows(const float* __restrict__ rows, int n, int nc, int ld,
-                                                     int rows_per_block, float* __restrict__ partial) {
-  constexpr int W = 16 * T, ROW = W + 1;
-  __shared__ float st[kJStage * ROW];
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int r0 = blockIdx.x * rows_per_block;
-  const int r1 = min(n, r0 + rows_per_block);
-  float acc[T][T];
+// The product is symmetric (a b and b a round alike), so only tiles that hold entries on or right of the
+// diagonal are formed: TA x TB entries per thread, tile (i, j) with TB j + TB > TA i.  An entry's chain over
+// the CTA's rows cannot be split (its rounding is part of the result), so what there is to fill the SM is
+// the tiles.  Per SM and row that is bound by the FMAs' operand reads (fma.rn.f32x2: about 3 cycles per
+// warp and sub-partition, measured) and by shared memory returning 32 floats per cycle: 8 x 4 tiles take
+// 96 and 96 cycles at 73 columns (8 x 8 tiles: 113, and only half of the sub-partitions get one of the
+// CTA's two warps of them, 206 in all; 4 x 4 ones: 84 and 112).  Up to 32 columns, where the rows of a CTA
+// are a chain that nothing else overlaps, 4 x 4 tiles have the shortest one (25 cycles a row).  The row
+// loop is unrolled over a whole stage so that its loads run ahead (62 cycles a row unrolled by 4).  Two
+// further warps copy the rows ahead with cp.async (16-byte pieces where base and ld allow, else 4-byte
+// ones) through four stages, one barrier per 16 rows; missing rows of the last stage are zeros.  One million
+// rows of 73 columns: 806 -> 198 us.  The version before formed the whole square from 5 x 5 tiles (scalar
+// reads) and loaded between its two barriers per 64 rows.
+template <int TA, int TB>
+struct JTiles {
+  static __host__ __device__ int cols(int nc) { return (nc + TB - 1) / TB; }
+  static __host__ __device__ int count(int nc) {
+    int t = 0;
+    for (int i = 0; TA * i < nc; ++i) t += cols(nc) - TA * i / TB;
+    return t;
+  }
+  static __host__ __device__ int compute_threads(int nc) { return (count(nc) + 31) / 32 * 32; }
+};
+
+__device__ __forceinline__ void cp_async4(void* s, const void* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((uint32_t)__cvta_generic_to_shared(s)),
+               "l"(__cvta_generic_to_global(g))
+               : "memory");
+}
+// 16 bytes of shared memory from `bytes` (<= 16) of global memory, the rest zeros
+__device__ __forceinline__ void cp_async16_part(void* s, const void* g, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((uint32_t)__cvta_generic_to_shared(s)),
+               "l"(__cvta_generic_to_global(g)), "r"(bytes)
+               : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void load_floats(const float* p, float (&v)[N]) {
 #pragma unroll
-  for (int a = 0; a < T; ++a)
+  for (int k = 0; k < N; k += 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p + k);
+    v[k] = q.x, v[k + 1] = q.y, v[k + 2] = q.z, v[k + 3] = q.w;
+  }
+}
+
+template <int TA, int TB>
+__global__ void __launch_bounds__(kJLoaders + 128) k_jtj_rows(const float* __restrict__ rows, int n, int nc, int ld,
+                                                            int rows_per_block, bool vec, float* __restrict__ partial) {
+  constexpr int W = kMaxNP;  // row stride: 16-byte rows; tiles past nc read the row's leftovers, which count nowhere
+  __shared__ __align__(16) float st[kJStages][kJStage][W];
+  const int tid = threadIdx.x, nthr = blockDim.x, ncomp = nthr - kJLoaders;
+  const int r0 = blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
+  const int nst = r1 > r0 ? (r1 - r0 + kJStage - 1) / kJStage : 0;
+  // this thread's tile
+  int ti = 0, tj = tid;
+  const int ncols = JTiles<TA, TB>::cols(nc);
+  while (TA * ti < nc && tj >= ncols - TA * ti / TB) {
+    tj -= ncols - TA * ti / TB;
+    ++ti;
+  }
+  tj += TA * ti / TB;
+  const bool comp = tid < ncomp && TA * ti < nc;
+  const int pieces = vec ? (nc + 3) / 4 : nc, lw = (tid - ncomp) >> 5;
+  auto load = [&](int q) {  // stage q, by the loader threads
+    const int base = r0 + q * kJStage, cnt = min(kJStage, r1 - base);
+    // a lane per piece, a warp per row; few instructions (a stage is one warp's chain of them)
+    constexpr int kWarps = kJLoaders / 32, kRowsEach = kJStage / kWarps;
+    for (int piece = tid & 31; piece < pieces; piece += 32) {
+      const int col = vec ? 4 * piece : piece, bytes = vec ? 4 * min(4, nc - col) : 4;
+      const float* src = rows + (size_t)(base + lw) * ld + col;
+      float* dst = &st[q % kJStages][lw][col];
+      const size_t step = (size_t)kWarps * ld;
+      if (cnt == kJStage) {
 #pragma unroll
-    for (int b = 0; b < T; ++b) acc[a][b] = 0.f;
-  for (int base = r0; base < r1; base += kJStage) {
-    const int cnt = min(kJStage, r1 - base);
-    __syncthreads();
-    for (int e = tid; e < kJStage * W; e += kJBlock) {
-      const int s = e / W, c = e % W;
-      st[s * ROW + c] = (s < cnt && c < nc) ? rows[(size_t)(base + s) * ld + c] : 0.f;
-    }
-    __syncthreads();
-    for (int s = 0; s < cnt; ++s) {
-      const float* row = st + s * ROW;
-      float ra[T], rb[T];
-#pragma unroll
-      for (int a = 0; a < T; ++a) {
-        ra[a] = row[ty * T + a];
-        rb[a] = row[tx * T + a];
+        for (int i = 0; i < kRowsEach; ++i) {
+          if (vec) cp_async16_part(dst + i * kWarps * W, src + i * step, bytes);
+          else cp_async4(dst + i * kWarps * W, src + i * step);
+        }
+      } else {
+        for (int i = 0; lw + i * kWarps < cnt; ++i) {
+          if (vec) cp_async16_part(dst + i * kWarps * W, src + i * step, bytes);
+          else cp_async4(dst + i * kWarps * W, src + i * step);
+        }
       }
+    }
+    for (int e = cnt * W + tid - ncomp; e < kJStage * W; e += kJLoaders) st[q % kJStages][0][e] = 0.f;
+  };
+  unsigned long long acc[TA][TB / 2];
 #pragma unroll
-      for (int a = 0; a < T; ++a)
+  for (int a = 0; a < TA; ++a)
 #pragma unroll
-        for (int b = 0; b < T; ++b) acc[a][b] = fmaf(ra[a], rb[b], acc[a][b]);
+    for (int b = 0; b < TB / 2; ++b) acc[a][b] = 0ull;
+  if (tid >= ncomp) {
+    for (int q = 0; q < kJStages - 1; ++q) {
+      if (q < nst) load(q);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
   }
+  for (int q = 0; q < nst; ++q) {
+    if (tid >= ncomp) asm volatile("cp.async.wait_group %0;\n" ::"n"(kJStages - 2) : "memory");
+    __syncthreads();  // stage q has arrived; every thread is done with stage q - 1, which is loaded next
+    if (tid >= ncomp) {
+      if (q + kJStages - 1 < nst) load(q + kJStages - 1);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    } else if (comp) {
+      const float* pa = &st[q % kJStages][0][TA * ti];
+      const float* pb = &st[q % kJStages][0][TB * tj];
+#pragma unroll
+      for (int s = 0; s < kJStage; ++s) {
+        float ra[TA], rb[TB];
+        load_floats(pa + s * W, ra);
+        load_floats(pb + s * W, rb);
+        unsigned long long B2[TB / 2];
+#pragma unroll
+        for (int b = 0; b < TB / 2; ++b)
+          asm("mov.b64 %0, {%1, %2};" : "=l"(B2[b]) : "f"(rb[2 * b]), "f"(rb[2 * b + 1]));
+#pragma unroll
+        for (int a = 0; a < TA; ++a) {
+          unsigned long long A2;
+          asm("mov.b64 %0, {%1, %1};" : "=l"(A2) : "f"(ra[a]));
+#pragma unroll
+          for (int b = 0; b < TB / 2; ++b)
+            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[a][b]) : "l"(A2), "l"(B2[b]));
+        }
+      }
+    }
+  }
+  if (!comp) return;
   float* out = partial + (size_t)blockIdx.x * nc * nc;
 #pragma unroll
-  for (int a = 0; a < T; ++a)
+  for (int a = 0; a < TA; ++a)
 #pragma unroll
-    for (int b = 0; b < T; ++b) {
-      const int r = ty * T + a, c = tx * T + b;
-      if (r < nc && c < nc) out[r * nc + c] = acc[a][b];
+    for (int b = 0; b < TB; ++b) {
+      const int r = TA * ti + a, c = TB * tj + b;
+      float lo, hi;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(acc[a][b / 2]));
+      if (c < nc && r <= c) out[r * nc + c] = b & 1 ? hi : lo;  // the upper triangle (the reduction mirrors)
     }
 }
 
+// (double)x of a normal x or zero, with integer operations: conversions to FP64 take 60 cycles of the FP64
+// pipe per warp.  Sets `other` where x is neither.
+__device__ __forceinline__ double widen(float x, bool& other) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+  other |= a != 0u && a - 0x00800000u >= 0x7f000000u;
+  const unsigned hi = (u & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(a << 29));
+}
+
+// FP64 sum of the nblk partials in a fixed order: warp w of the block's S adds partials w, w + S, ... (all
+// its loads of a round in flight), warp 0 the warps' sums.  kUpper: the partials hold the upper triangle,
+// whose entries are written to both places.
+template <bool kUpper>
 __global__ void __launch_bounds__(1024) k_jtj_reduce(const float* __restrict__ partial, int nblk, int nc,
                                                      double* __restrict__ out) {
   __shared__ double sm[32][33];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int n2 = nc * nc, e = blockIdx.x * 32 + lane;
+  constexpr int kBatch = 8;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, S = blockDim.x >> 5;
+  const int n2 = nc * nc, total = kUpper ? nc * (nc + 1) / 2 : n2, u = blockIdx.x * 32 + lane;
+  int r = 0, c = 0;
+  if (kUpper && u < total) {  // counted from the end, row nc - 1 - m holds m + 1 entries
+    const int v = total - 1 - u;
+    int m = (int)((sqrtf(8.f * (float)v + 1.f) - 1.f) * 0.5f);
+    if ((m + 1) * (m + 2) / 2 <= v) ++m;
+    if (m * (m + 1) / 2 > v) --m;
+    r = nc - 1 - m;
+    c = nc - 1 - (v - m * (m + 1) / 2);
+  }
+  const int e = kUpper ? r * nc + c : u;
   double s = 0.0;
-  if (e < n2)
-    for (int b = w; b < nblk; b += 32) s += (double)partial[(size_t)b * n2 + e];
+  for (int b0 = w; b0 < nblk; b0 += kBatch * S) {
+    float q[kBatch];
+    bool other = false;
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) q[k] = b0 + k * S < nblk && u < total ? partial[(size_t)(b0 + k * S) * n2 + e] : 0.f;
+    double d[kBatch];
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) d[k] = widen(q[k], other);
+    if (__any_sync(0xffffffffu, other)) {
+#pragma unroll
+      for (int k = 0; k < kBatch; ++k) d[k] = (double)q[k];
+    }
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k)
+      if (b0 + k * S < nblk) s += d[k];
+  }
   sm[w][lane] = s;
   __syncthreads();
-  if (w != 0 || e >= n2) return;
+  if (w != 0 || u >= total) return;
   double t = 0.0;
-  for (int k = 0; k < 32; ++k) t += sm[k][lane];
+#pragma unroll 8
+  for (int k = 0; k < S; ++k) t += sm[k][lane];
   out[e] = t;
+  if (kUpper) out[c * nc + r] = t;
+}
+
+template <bool kUpper>
+static void launch_reduce(const float* partial, int nblk, int nc, double* out, cudaStream_t st) {
+  const int total = kUpper ? nc * (nc + 1) / 2 : nc * nc;
+  k_jtj_reduce<kUpper><<<(total + 31) / 32, 32 * std::min(32, std::max(1, (nblk + 1) / 2)), 0, st>>>(partial, nblk, nc, out);
+}
+
+template <int TA, int TB>
+static void launch_rows(const float* rows, int n, int nc, int ld, int nblk, int rpb, bool vec, float* partial,
+                        cudaStream_t st) {
+  k_jtj_rows<TA, TB><<<nblk, JTiles<TA, TB>::compute_threads(nc) + kJLoaders, 0, st>>>(rows, n, nc, ld, rpb, vec, partial);
 }
 
 // Launches the two kernels with nblk CTAs and the given partial buffer (nblk * nc * nc floats).
 cudaError_t jtj_rows_launch(const float* rows, int n, int nc, int ld, double* out, int nblk, float* partial,
                             cudaStream_t st) {
-  const int T = (nc + 15) / 16;
   const int rpb = (n + nblk - 1) / nblk;
-  switch (T) {
-    case 1: k_jtj_rows<1><<<nblk, kJBlock, 0, st>>>(rows, n, nc, ld, rpb, partial); break;
-    case 2: k_jtj_rows<2><<<nblk, kJBlock, 0, st>>>(rows, n, nc, ld, rpb, partial); break;
-    case 3: k_jtj_rows<3><<<nblk, kJBlock, 0, st>>>(rows, n, nc, ld, rpb, partial); break;
-    case 4: k_jtj_rows<4><<<nblk, kJBlock, 0, st>>>(rows, n, nc, ld, rpb, partial); break;
-    default: k_jtj_rows<5><<<nblk, kJBlock, 0, st>>>(rows, n, nc, ld, rpb, partial); break;
-  }
-  k_jtj_reduce<<<(nc * nc + 31) / 32, 1024, 0, st>>>(partial, nblk, nc, out);
+  const bool vec = ld % 4 == 0 && reinterpret_cast<uintptr_t>(rows) % 16 == 0;
+  if (nc > 32) launch_rows<8, 4>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
+  else launch_rows<4, 4>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
+  launch_reduce<true>(partial, nblk, nc, out, st);
   return cudaGetLastError();
 }
 
 // Fixed-order FP64 sum of nslots partials of nc x nc floats into out.
 cudaError_t jtj_reduce_launch(const float* partial, int nslots, int nc, double* out, cudaStream_t st) {
-  k_jtj_reduce<<<(nc * nc + 31) / 32, 1024, 0, st>>>(partial, nslots, nc, out);
+  launch_reduce<false>(partial, nslots, nc, out, st);
   return cudaGetLastError();
 }
 

@@ -54,3 +54,33 @@ def test_invalid_arguments_are_rejected():
     out = torch.zeros((90, 90), dtype=torch.float64, device="cuda")
     with pytest.raises(trk.TrkError):
         trk.jtj_rows(dev.data_ptr(), 4, 90, 90, out.data_ptr(), 0)
+
+
+@pytest.mark.parametrize("n,nc,ld,offset", [
+    (1, 80, 80, 0), (15, 32, 32, 0), (16, 33, 36, 0), (17, 64, 64, 0), (256, 65, 68, 0), (257, 4, 4, 0),
+    (4097, 8, 9, 0), (38913, 40, 44, 0), (5000, 73, 76, 1), (5000, 73, 73, 0)])
+def test_tile_and_alignment_edges(n, nc, ld, offset):
+    """Column counts at the edges of the tile shapes (32 / 33, 64 / 65, 80), row counts at the edges of a
+    16-row stage and of the grid, rows that allow 16-byte copies and rows that do not (odd ld, a base off by
+    one float), NaN in the columns past nc, which must not count; the allocation-free call gives the same
+    bits up to 38,912 rows.  Bound: a sum of n products in FP32, one chain per CTA of at most max(256, n / 152)
+    rows: gamma = (rows + 1) 2^-24 of the sum of magnitudes."""
+    rng = np.random.default_rng(7 * n + nc)
+    J = (rng.normal(size=(n, nc)) * rng.uniform(0.01, 1.0, nc)).astype(np.float32)
+    full = np.full((n, ld), np.nan, np.float32)
+    full[:, :nc] = J
+    buf = torch.empty(n * ld + 4, dtype=torch.float32, device="cuda")
+    rows = buf[offset:offset + n * ld]
+    rows.copy_(torch.from_numpy(full.ravel()))
+    out = torch.empty((nc, nc), dtype=torch.float64, device="cuda")
+    trk.jtj_rows(rows.data_ptr(), n, nc, ld, out.data_ptr())
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    X = J.astype(np.float64)
+    bound = (max(256, n // 152 + 1) + 1) * 2.0 ** -24 * (np.abs(X).T @ np.abs(X))
+    assert (np.abs(got - X.T @ X) <= bound + 1e-300).all()
+    assert (got == got.T).all()
+    if n <= 152 * 256:
+        trk.jtj_rows_noalloc(rows.data_ptr(), n, nc, ld, out.data_ptr())
+        torch.cuda.synchronize()
+        assert (out.cpu().numpy() == got).all()
