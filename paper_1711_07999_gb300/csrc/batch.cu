@@ -48,7 +48,7 @@ struct trk_batch {
   int pose_iters = 0, shape_iters = 0, shape_sweeps = 0, precision = 0, shape_solver = 0;
   int max_links = 0, max_np = 0;
   int assoc_blocks = kAssocBlocksPerSM * 152;  // persistent association blocks
-  int tail_blocks = 304;      // association-tail blocks (shared by all sessions' queues)
+  int tail_blocks = kTailBlocksPerSM * 152;  // association-tail blocks (shared by all sessions' queues)
   Dev* d_devs = nullptr;
   unsigned* d_ctl = nullptr;  // [0] association units of the frame, [1] unused, [2] tail counter
   unsigned* d_prefix = nullptr;  // [n + 1] queued pixels before each session
@@ -463,7 +463,7 @@ trk_status batch_step_launch(BatchStep* bs, trk_session* const* ss, int n, const
   v.precision = p0.precision;
   v.max_links = max_links;
   v.assoc_blocks = kAssocBlocksPerSM * 152;
-  v.tail_blocks = 2 * 152;
+  v.tail_blocks = kTailBlocksPerSM * 152;
   v.d_devs = reinterpret_cast<const Dev*>(dbuf + o_devs);
   for (int k = 0; k < kKinds; ++k) {
     v.tables[k].n = (int)maps[k].size();
@@ -491,7 +491,7 @@ trk_status batch_step_launch(BatchStep* bs, trk_session* const* ss, int n, const
 extern "C" {
 
 trk_status trk_batch_create(trk_session* const* sessions, int32_t n_sessions, trk_batch** out) {
-  return batch_create(sessions, n_sessions, 4 * 152, 2 * 152, out);
+  return batch_create(sessions, n_sessions, kAssocBlocksPerSM * 152, kTailBlocksPerSM * 152, out);
 }
 
 trk_status trk_batch_track_device(trk_batch* b, const float* const* d_depths, void* cuda_stream) {

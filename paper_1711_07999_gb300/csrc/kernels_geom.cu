@@ -43,6 +43,7 @@ __device__ __forceinline__ void skin_impl(const Dev& d, BlockPos bp, int phi_buf
     d.zbuf[k] = ~0ull;
     d.head[k] = -1;
   }
+  for (int k = tid, n = d.cam.H * occ_row(d.cam.W); k < n; k += stride) d.occ[k] = 0u;
   for (int k = tid; k < d.V; k += stride) d.acc[k] = Acc4{0, 0, 0, 0};
   if (tid == 0) {
     d.stats[0] = 0;
@@ -195,7 +196,10 @@ __device__ __forceinline__ void visibility_impl(const Dev& d, BlockPos bp) {
         d.rec[i] = make_float4(pl.x, pl.y, pl.z, __int_as_float(old));
         // the first vertex of a bucket is also stored with the pixel, so that a bucket holding one vertex
         // is read with two independent loads (head, pixrec) instead of a dependent chain
-        if (old < 0) d.pixrec[k] = make_float4(pl.x, pl.y, pl.z, __int_as_float(i));
+        if (old < 0) {
+          d.pixrec[k] = make_float4(pl.x, pl.y, pl.z, __int_as_float(i));
+          atomicOr(&d.occ[(int)fv * occ_row(c.W) + ((int)fu >> 5)], 1u << ((int)fu & 31));
+        }
       }
     }
   }
@@ -346,48 +350,75 @@ __device__ __forceinline__ float3 back_project(const Cam& c, int px, int py, flo
                      (float)((double)dep - (double)c.oz));
 }
 
+// The pixel's point, once per frame for its twelve or so iterations: on this GPU the ~20 FP64 operations and
+// conversions of a back-projection occupy the FP64 pipe for ~1,250 cycles per warp.
+__device__ __forceinline__ void store_point(const Dev& d, int px, int py, int k, float z) {
+  const float3 p = back_project(d.cam, px, py, z);
+  d.ppos[k] = make_float4(p.x, p.y, p.z, z);
+}
+
 // One lane's pixel (px, py) of a warp's unit (active false: the lane has none; it still takes part in
 // the warp's votes).
 __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, bool active) {
-  const Cam c = d.cam;
+  const Cam& c = d.cam;
   const int lane = threadIdx.x & 31;
   const bool inimg = active && px < c.W && py < c.H;
   const int k = py * c.W + px;
-  const float dep = inimg ? d.depth[k] : 0.f;
   const float tau2 = c.tau * c.tau;
   Best best{-1, 0.f, make_float3(0.f, 0.f, 0.f)};
   float3 p = make_float3(0.f, 0.f, 0.f);
   bool open = false;
-  if (dep > 0.f && d.association == 1) {
-    // the nearest corner of the triangle the z-buffer holds at this pixel (O(1), no queue)
-    p = back_project(c, px, py, dep);
-    const unsigned long long key = d.zbuf[k];
-    if (key != ~0ull) {
-      const int4 t = d.tris[(int)(unsigned)(key & 0xffffffffu)];
-      consider(t.x, p, d.v[t.x], tau2, best);
-      consider(t.y, p, d.v[t.y], tau2, best);
-      consider(t.z, p, d.v[t.z], tau2, best);
-    }
-  } else if (dep > 0.f) {
-    p = back_project(c, px, py, dep);
-    open = true;
-    if (c.R == 0) {
+  if (inimg) {  // (the units list pixels with a valid depth)
+    const float4 pp = d.ppos[k];
+    p = f3(pp);
+    const float dep = pp.w;
+    if (d.association == 1) {
+      // the nearest corner of the triangle the z-buffer holds at this pixel (O(1), no queue)
+      const unsigned long long key = d.zbuf[k];
+      if (key != ~0ull) {
+        const int4 t = d.tris[(int)(unsigned)(key & 0xffffffffu)];
+        consider(t.x, p, d.v[t.x], tau2, best);
+        consider(t.y, p, d.v[t.y], tau2, best);
+        consider(t.z, p, d.v[t.z], tau2, best);
+      }
+    } else if (c.R == 0) {
       const int q0[1] = {k};
       scan_group<1, false>(d, q0, p, tau2, best);
-      open = false;
     } else {
-      // rings 0 and 1 (9 buckets) in two rounds of independent loads: the pixel's own bucket with the
-      // first four of ring 1, then the other four; the ring-1 bound decides whether the search goes on
-      int q[5];
+      // rings 0 and 1 (9 buckets): the heads and first records of the pixel's own bucket and the first four
+      // of ring 1 are loaded together; where the own bucket holds a vertex nearer than anything outside it
+      // can be (several vertices per pixel: meshes finer than the image), that is the answer and the lists of
+      // the others are not walked; else they are, with the other four buckets after them, and the ring-1 bound
+      // decides whether the search goes on
+      int q[5], h[5], first[5];
       q[0] = k;
 #pragma unroll
       for (int u = 0; u < 4; ++u) q[1 + u] = ring_bucket(px, py, 1, u, c.W, c.H);
-      scan_group<5, false>(d, q, p, tau2, best);
+      {
+        float4 f[5];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = ring_bucket(px, py, 1, 4 + u, c.W, c.H);
-      scan_group<4, false>(d, q, p, tau2, best);
-      const float lb = dep * (1.0f + 0.499f) * c.kappa;
-      if (lb > c.tau || (best.i >= 0 && lb * lb > best.d2) || c.R == 1) open = false;
+        for (int u = 0; u < 5; ++u) {
+          h[u] = q[u] >= 0 ? __ldg(&d.head[q[u]]) : -1;
+          f[u] = q[u] >= 0 ? d.pixrec[q[u]] : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+        }
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+          first[u] = __float_as_int(f[u].w);
+          if (h[u] >= 0) consider(first[u], p, f[u], tau2, best);
+        }
+      }
+      if (h[0] >= 0) scan_rest(d, h[0], first[0], p, tau2, best);
+      const float lb0 = dep * 0.499f * c.kappa;
+      if (!(best.i >= 0 && lb0 * lb0 > best.d2)) {
+#pragma unroll
+        for (int u = 1; u < 5; ++u)
+          if (h[u] >= 0) scan_rest(d, h[u], first[u], p, tau2, best);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = ring_bucket(px, py, 1, 4 + u, c.W, c.H);
+        scan_group<4, false>(d, q, p, tau2, best);
+        const float lb = dep * (1.0f + 0.499f) * c.kappa;
+        open = !(lb > c.tau || (best.i >= 0 && lb * lb > best.d2) || c.R == 1);
+      }
     }
   }
   // queue the open pixels (one atomic per warp)
@@ -395,7 +426,7 @@ __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, boo
   unsigned base = 0;
   if (lane == 0 && om) base = atomicAdd(&d.qctl[0], __popc(om));
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int4(k, best.i, __float_as_int(best.d2), 0);
+  if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int2(k, best.i);
   if (inimg && !open) d.corr[k] = best.i;
   const bool done = !open && best.i >= 0;
   if (done) commit_pixel(d, best.i, p, best.v);
@@ -416,31 +447,67 @@ constexpr int kBatchTailPerLane = 4;  // ... and buckets each of them loads at o
 // correspondence (its first lane writes it and adds the pixel's sums).
 // One session's tail takes a warp per pixel (its queue is short and its latency is the slowest pixel's
 // rings); a batch's takes 8 lanes per pixel (four pixels per warp: throughput over many queues).
-template <int GL, int PL>
+//
+// A batch's lanes (kRows) take a row of the square each instead and read which of its buckets hold a vertex from
+// the occupancy bits, three words for the rings of a round together, so that an empty bucket -- most of
+// them at silhouettes and where the mesh is coarser than the image -- costs no load; a round takes rings
+// r0 .. r0 + 1 first, four more rings after that.
+template <int GL, int PL, bool kRows>
 __device__ __forceinline__ bool tail_item(const Dev& d, unsigned item, int gl, unsigned gmask) {
-  const Cam c = d.cam;
+  const Cam& c = d.cam;
   const float tau2 = c.tau * c.tau;
-  const int4 e = d.queue[item];
-  const int k = e.x, px = k % c.W, py = k / c.W;
-  const float dep = d.depth[k];
-  const float3 p = back_project(c, px, py, dep);
-  unsigned long long key = key_of(e.y, __int_as_float(e.z));
+  const int2 e = d.queue[item];
+  const int k = e.x, W = c.W, H = c.H, px = k % W, py = k / W;
+  const float4 pp = d.ppos[k];
+  const float dep = pp.w;
+  const float3 p = f3(pp);
   Best w{-1, 0.f, make_float3(0.f, 0.f, 0.f)};
-  // rings r0..r1 at a time, as many whole rings as the group's load slots hold (at least one): scanning
-  // rings past the one whose bound ends the search only confirms the argmin, so the result is the same
-  constexpr int kSlots = GL * PL;
+  if (e.y >= 0) consider(e.y, p, d.v[e.y], tau2, w);  // the nearest so far (its record's bits)
+  unsigned long long key = key_of(w.i, w.d2);
+  // several rings at a time: scanning rings past the one whose bound ends the search only confirms the
+  // argmin, so the result is the same
   for (int r0 = kRingsPerThread + 1; r0 <= c.R;) {
-    int r1 = r0, nb = 8 * r0;
-    while (r1 < c.R && nb + 8 * (r1 + 1) <= kSlots) nb += 8 * ++r1;
-    for (int t0 = 0; t0 < nb; t0 += kSlots) {
-      int q[PL];
+    int r1 = r0;
+    if constexpr (kRows) {
+      r1 = min(c.R, r0 == kRingsPerThread + 1 ? r0 + 1 : r0 + 3);
+      const int xs = max(0, px - r1), n = min(W - 1, px + r1) - xs + 1;
+      const int seen = px - r0 + 1 - xs, nseen = 2 * r0 - 1;  // the columns of the square already searched
+      for (int t = gl; t <= 2 * r1; t += GL) {
+        const int y = py + t - r1;
+        if (y < 0 || y >= H) continue;
+        const unsigned* row = d.occ + (size_t)y * occ_row(W) + (xs >> 5);
+        const int sh = xs & 31;
+        const unsigned w0 = row[0], w1 = row[1], w2 = row[2];
+        unsigned long long bits = __funnelshift_r(w0, w1, sh) | (unsigned long long)__funnelshift_r(w1, w2, sh) << 32;
+        bits &= ~0ull >> (64 - n);  // (1 <= n <= 63)
+        if (y > py - r0 && y < py + r0) {
+          const unsigned long long m = (1ull << nseen) - 1;
+          bits &= ~(seen >= 0 ? m << seen : m >> -seen);
+        }
+        while (bits) {
+          int q[PL];
 #pragma unroll
-      for (int u = 0; u < PL; ++u) {
-        int t = t0 + gl + GL * u, r = r0;
-        while (t < nb && t >= 8 * r) t -= 8 * r++;  // bucket t of the group: ring r, position t
-        q[u] = t0 + gl + GL * u < nb ? ring_bucket(px, py, r, t, c.W, c.H) : -1;
+          for (int u = 0; u < PL; ++u) {
+            q[u] = bits ? y * W + xs + __ffsll((long long)bits) - 1 : -1;
+            bits &= bits - 1;
+          }
+          scan_group<PL, true>(d, q, p, tau2, w);
+        }
       }
-      scan_group<PL, true>(d, q, p, tau2, w);
+    } else {
+      constexpr int kSlots = GL * PL;  // as many whole rings as the group's load slots hold (at least one)
+      int nb = 8 * r0;
+      while (r1 < c.R && nb + 8 * (r1 + 1) <= kSlots) nb += 8 * ++r1;
+      for (int t0 = 0; t0 < nb; t0 += kSlots) {
+        int q[PL];
+#pragma unroll
+        for (int u = 0; u < PL; ++u) {
+          int t = t0 + gl + GL * u, r = r0;
+          while (t < nb && t >= 8 * r) t -= 8 * r++;  // bucket t of the group: ring r, position t
+          q[u] = t0 + gl + GL * u < nb ? ring_bucket(px, py, r, t, W, H) : -1;
+        }
+        scan_group<PL, true>(d, q, p, tau2, w);
+      }
     }
     unsigned long long kk = key_of(w.i, w.d2);
     kk = kk < key ? kk : key;
@@ -466,8 +533,8 @@ __device__ __forceinline__ bool tail_item(const Dev& d, unsigned item, int gl, u
 }
 
 // Persistent warps take the frame's association units (up to 32 pixels of a tile with a valid depth; one
-// session's from k_tiles, a batch's from the depth gather), warp w the units w, w + (warps in the grid),
-// ...: no counter and no block barrier, so a warp whose pixels are cheap goes on to its next unit at once,
+// session's from k_tiles, a batch's from the depth gather), warp w of block b the units w G + b (G blocks: a
+// short list spreads over all SMs), then every (warps in the grid)-th: no counter and no block barrier, so a warp whose pixels are cheap goes on to its next unit at once,
 // and the interleaving spreads the units of costly sessions over all warps.  In a batch each warp keeps
 // its own copy of its unit's session descriptor in shared memory (reloaded when the session changes).
 // Pixels outside the units keep the "no correspondence" the frame's depth copy wrote.
@@ -481,7 +548,7 @@ __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const D
   const unsigned nw = gridDim.x * (kBlock / 32);
   if (single) {
 #pragma unroll 1
-    for (unsigned u = blockIdx.x * (kBlock / 32) + w; u < n; u += nw) {
+    for (unsigned u = w * gridDim.x + blockIdx.x; u < n; u += nw) {
       const int4 h = *reinterpret_cast<const int4*>(&list[u]);  // (session, x0, y0, pixels)
       const int o = lane < h.w ? list[u].off[lane] : 0;
       associate_impl(d0, h.y + (o & 15), h.z + (o >> 4), lane < h.w);
@@ -490,7 +557,7 @@ __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const D
   }
   int cur = -1;
 #pragma unroll 1
-  for (unsigned u = blockIdx.x * (kBlock / 32) + w; u < n; u += nw) {
+  for (unsigned u = w * gridDim.x + blockIdx.x; u < n; u += nw) {
     const int4 h = *reinterpret_cast<const int4*>(&list[u]);
     const int o = lane < h.w ? list[u].off[lane] : 0;
     if (h.x != cur) {
@@ -513,7 +580,7 @@ __global__ void __launch_bounds__(32 * kTailWarps) k_associate_tail(Dev d) {
   const unsigned warps = gridDim.x * kTailWarps;  // warp w takes entry w first, then the counter's
   int done = 0;
   for (unsigned item = blockIdx.x * kTailWarps + (threadIdx.x >> 5); item < n;) {
-    done += tail_item<32, kTailPerLane>(d, item, gl, gmask);
+    done += tail_item<32, kTailPerLane, false>(d, item, gl, gmask);
     if (warps >= n) break;
     unsigned next = 0;
     if (gl == 0) next = warps + atomicAdd(&d.qctl[1], 1u);
@@ -552,7 +619,7 @@ __global__ void __launch_bounds__(1024) k_tail_prefix(const Dev* devs, int n_ses
 // A batch: the lane groups take entries of the concatenated queues of all sessions, group g the g-th, then
 // the rest from one counter; an entry's session is found in the prefix and its descriptor read through
 // the cache.
-__global__ void __launch_bounds__(32 * kTailWarps) k_associate_tail_batch(const Dev* devs, int n_sessions,
+__global__ void __launch_bounds__(32 * kTailWarps, kTailBlocksPerSM) k_associate_tail_batch(const Dev* devs, int n_sessions,
                                                                           const unsigned* prefix, unsigned* ctl) {
   constexpr int GL = kBatchTailLanes;
   const int lane = threadIdx.x & 31, gl = lane % GL, gbase = lane - gl;
@@ -566,7 +633,10 @@ __global__ void __launch_bounds__(32 * kTailWarps) k_associate_tail_batch(const 
       if (prefix[mid] <= item) lo = mid; else hi = mid - 1;
     }
     const Dev& d = devs[lo];
-    if (tail_item<GL, kBatchTailPerLane>(d, item - prefix[lo], gl, gmask) && gl == 0) atomicAdd(&d.stats[0], 1);
+    // (the row windows of the occupancy bits hold up to 63 columns)
+    const bool got = d.cam.R <= 31 ? tail_item<GL, kBatchTailPerLane, true>(d, item - prefix[lo], gl, gmask)
+                                   : tail_item<GL, kBatchTailPerLane, false>(d, item - prefix[lo], gl, gmask);
+    if (got && gl == 0) atomicAdd(&d.stats[0], 1);
     if (groups >= total) break;
     unsigned next = 0;
     if (gl == 0) next = groups + atomicAdd(&ctl[2], 1u);
@@ -623,6 +693,7 @@ __global__ void __launch_bounds__(kBlock) k_tiles(Dev d, const float* __restrict
     const_cast<float*>(d.depth)[k] = z;
     d.corr[k] = -1;
     valid = z > 0.f;
+    if (valid) store_point(d, px, py, k, z);
   }
   list_units(valid, 0, tx, ty, d.units, &d.qctl[2]);
 }
@@ -664,6 +735,7 @@ __global__ void __launch_bounds__(kBlock) k_gather_depth_b(BatchGrid g, const fl
     const_cast<float*>(d.depth)[k] = z;
     d.corr[k] = -1;
     valid = z > 0.f;
+    if (valid) store_point(d, px, py, k, z);
   }
   list_units(valid, m.x, m.y, m.z, units, &ctl[0]);
 }

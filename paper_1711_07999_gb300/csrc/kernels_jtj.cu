@@ -17,7 +17,7 @@ namespace trk {
 constexpr int kJBlock = 256;      // rows that make a CTA worth having (the grid's rule)
 constexpr int kJStage = 16;       // rows per pipeline stage
 constexpr int kJStages = 4;
-constexpr int kJLoaders = 64;     // threads that only load
+constexpr int kJLoaders = 128;    // threads that only load
 constexpr int kJMaxBlocks = 296;
 
 // The product is symmetric (a b and b a round alike), so only tiles that hold entries on or right of the

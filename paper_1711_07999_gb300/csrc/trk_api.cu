@@ -535,7 +535,8 @@ void carve_all(trk_session* s) {
   carve(s, &d.lm_ok, 2 * kCandidates);
   carve(s, &d.v, V); carve(s, &d.n, V); carve(s, &d.fn, F); carve(s, &d.rec, V);
   carve(s, &d.head, npx); carve(s, &d.zbuf, npx); carve(s, &d.corr, npx);
-  carve(s, &d.pixrec, npx); carve(s, &d.queue, npx); carve(s, &d.qctl, 4);
+  carve(s, &d.pixrec, npx); carve(s, &d.queue, npx); carve(s, &d.qctl, 4); carve(s, &d.ppos, npx);
+  carve(s, &d.occ, (size_t)d.cam.H * occ_row(d.cam.W));
   carve(s, &d.units, (size_t)kUnitsPerTile * ((d.cam.W + 15) / 16) * ((d.cam.H + 15) / 16));
   carve(s, &d.acc, V); carve(s, &d.vispix, V); carve(s, &d.rg, V); carve(s, &d.phi0, V);
   carve(s, &dadj_off, V + 1); carve(s, &dadj, s->hm.adj.size());
@@ -1150,6 +1151,7 @@ trk_status trk_step_visibility(trk_session* s) {
   NEED_RESIDENT(s);
   // empty buckets first, so that calling this step twice cannot insert a vertex twice
   CK(cudaMemsetAsync(s->d.head, 0xFF, sizeof(int) * s->d.cam.W * s->d.cam.H, s->stream));
+  CK(cudaMemsetAsync(s->d.occ, 0, sizeof(unsigned) * s->d.cam.H * occ_row(s->d.cam.W), s->stream));
   launch_visibility(s->d, s->stream);
   return sync_check(s);
 }

@@ -22,6 +22,7 @@ constexpr int kMaxNP = 80;
 constexpr int kMaxJtjGroup = 4;    // vertex blocks of 256 per [J r] block at most (trk_params.jtj_group)
 constexpr int kUnitsPerTile = 8;   // association units (16 x 2 pixels) per 16 x 16 tile
 constexpr int kAssocBlocksPerSM = 4;  // resident association blocks per SM (registers sized for it)
+constexpr int kTailBlocksPerSM = 3;   // the same of a batch's association tail
 constexpr int kCandidates = 6;      // damping values tried per LM iteration: lambda * 10^c, c = 0..5
 constexpr float kFix = 1073741824.0f;  // 2^30: fixed-point scale of the per-vertex sums
 
@@ -310,6 +311,10 @@ inline S set_error(S st, const char* msg) { return static_cast<S>(set_error_code
 
 namespace trk {
 
+// Words per row of the bucket occupancy bits: two more than the row's, so that a window of up to 64 bits is read
+// as three words from its first.
+__host__ __device__ inline int occ_row(int W) { return (W + 31) / 32 + 2; }
+
 // A warp's share of the association: up to 32 pixels of one 16 x 16 tile that hold a valid depth, in
 // row-major order (lane l takes pixel (x0 + off[l] % 16, y0 + off[l] / 16) for l < n).
 struct __align__(16) AssocUnit {
@@ -354,7 +359,9 @@ struct Dev {
   float4* rec;
   float4* pixrec;  // [W*H] first vertex inserted into each pixel's bucket: x, y, z, index bits
   int* head;
-  int4* queue;     // [W*H] pixels whose association search continues past the thread-owned rings
+  unsigned* occ;   // [H][occ_row(W)] one bit per pixel: its bucket holds a vertex
+  float4* ppos;    // [W*H] pixels with a valid depth: back-projected point (session-local frame), depth in w
+  int2* queue;     // [W*H] pixels whose association search goes on past the thread-owned rings: (pixel, nearest so far)
   unsigned int* qctl;  // [0] queued pixels, [1] next queue entry to take, [2] association units, [3] unused
   AssocUnit* units;  // [8 ceil(W/16) ceil(H/16)] association units of the frame (up to 32 valid pixels of a tile)
   unsigned long long* zbuf;
