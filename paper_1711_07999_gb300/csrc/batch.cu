@@ -59,6 +59,8 @@ struct trk_batch {
   cudaEvent_t src_ev[4] = {};      // the copy out of each slot has been done
   int src_slot = 0;
   cudaStream_t cap = nullptr;
+  ForkStreams fork;  // of the capture (the graph's parallel branches); made where there are several tile classes
+  bool has_fork = false;
   cudaGraphExec_t graph = nullptr;
 };
 
@@ -109,6 +111,7 @@ struct FrameView {
   AssocUnit* d_tiles = nullptr;     // [kUnitsPerTile tables[kAssoc].n]
   const float* const* d_srcs = nullptr;  // [B] depth of each session (device-readable)
   const Dev* const* host_devs = nullptr;  // [B] the sessions' descriptors on the host
+  const ForkStreams* fork = nullptr;      // side streams of the capture
   int reduce_threads = 32;                // the reduction's block: the largest need of the sessions
 };
 
@@ -142,7 +145,7 @@ void enqueue_frame_view(const FrameView& v, cudaStream_t st) {
     }
     NvtxRange nv("normal equations, LM step");
     launch_normal_equations_b(gj, nj, grid_of(v, kReduce), v.tables[kReduce].n, L, v.precision, cur, it, st,
-                              v.reduce_threads);
+                              v.reduce_threads, v.fork);
     launch_lm_b(grid_of(v, kLm), v.tables[kLm].n, grid_of(v, kRows), v.tables[kRows].n, L, cur, st);
   }
   for (int it = 0; it < S; ++it) {
@@ -176,6 +179,7 @@ FrameView view_of(const trk_batch* b, const std::vector<const Dev*>& host_devs) 
   v.d_srcs = b->d_srcs;
   v.host_devs = host_devs.data();
   v.reduce_threads = reduce_threads_for(host_devs.data(), v.B);
+  v.fork = b->has_fork ? &b->fork : nullptr;
   return v;
 }
 
@@ -189,6 +193,11 @@ void free_batch(trk_batch* b) {
   if (!b) return;
   if (b->graph) cudaGraphExecDestroy(b->graph);
   if (b->cap) cudaStreamDestroy(b->cap);
+  for (cudaStream_t s : b->fork.side)
+    if (s) cudaStreamDestroy(s);
+  for (cudaEvent_t e : b->fork.join)
+    if (e) cudaEventDestroy(e);
+  if (b->fork.fork) cudaEventDestroy(b->fork.fork);
   for (Table& t : b->tables) cudaFree(t.d_map);
   cudaFree(b->d_devs);
   cudaFree(b->d_ctl);
@@ -299,6 +308,16 @@ trk_status batch_create(trk_session* const* sessions, int n_sessions, int assoc_
   BCK(cudaMallocHost(&b->h_srcs, sizeof(float*) * devs.size() * kSrcSlots));
   for (cudaEvent_t& e : b->src_ev) BCK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   BCK(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
+  int classes = 0;
+  for (int t = kJtj1; t <= kJtj5; ++t) classes += b->tables[t].n > 0;
+  if (classes > 1) {
+    BCK(cudaEventCreateWithFlags(&b->fork.fork, cudaEventDisableTiming));
+    for (int k = 0; k + 1 < classes; ++k) {
+      BCK(cudaStreamCreateWithFlags(&b->fork.side[k], cudaStreamNonBlocking));
+      BCK(cudaEventCreateWithFlags(&b->fork.join[k], cudaEventDisableTiming));
+    }
+    b->has_fork = true;
+  }
   cudaGraph_t g = nullptr;
   BCK(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
   enqueue_batch_frame(b, b->cap);

@@ -41,12 +41,14 @@ __device__ __forceinline__ float3 Lfun(float4 c, float4 h) {
 // The block's rows (compacted to A) are staged in shared memory; 16 x 16 threads each own a TxT tile
 // of the (16T) x (16T) product and sweep the rows.
 // ---------------------------------------------------------------------------------------------
-// Copies the link tables this block needs (H_Delta, Xi, parents) to shared memory.
-__device__ __forceinline__ void load_link_tables(const Dev& d, DQ* sHd, float* sXi, int* sPar) {
-  for (int j = threadIdx.x; j < d.L; j += kBlock) {
-    sHd[j] = d.Hd[j];
-    for (int c = 0; c < 6; ++c) sXi[6 * j + c] = d.xi[8 * j + c];
-    sPar[j] = d.links->parent[j];
+// Copies the link tables this block needs to shared memory: H_Delta, and per link eight floats (the twist
+// Xi, the parent's index as bits, unused), read as two 16-byte pieces in the Jacobian's walk.
+__device__ __forceinline__ void load_link_tables(const Dev& d, DQ* sHd, float* sXi) {
+  for (int t = threadIdx.x; t < 2 * d.L; t += kBlock) {
+    reinterpret_cast<float4*>(sHd)[t] = reinterpret_cast<const float4*>(d.Hd)[t];
+    float4 x = reinterpret_cast<const float4*>(d.xi)[t];
+    if (t & 1) x.z = __int_as_float(d.links->parent[t >> 1]);
+    reinterpret_cast<float4*>(sXi)[t] = x;
   }
 }
 
@@ -98,7 +100,7 @@ __device__ __forceinline__ int block_rows(const Dev& d, int blk, int row_base, i
 // [0, width) with width >= NP, zero beyond NP) and sets r2 = r_i^2 (0 outside A).  The link tables must
 // be in shared memory; the caller synchronises before reading Js.
 __device__ __forceinline__ void jacobian_row(const Dev& d, const RowSlot& rs, int phi_buf, float* Js, int ROW,
-                                             int width, const DQ* sHd, const float* sXi, const int* sPar, float& r2) {
+                                             int width, const DQ* sHd, const float* sXi, float& r2) {
   r2 = 0.f;
   if (!rs.inA) return;
   const Acc4 a4 = rs.a4;
@@ -197,14 +199,16 @@ __device__ __forceinline__ void jacobian_row(const Dev& d, const RowSlot& rs, in
 #pragma unroll
     for (int c = 0; c < 6; ++c) E[c] = es[0][c];
     pop();
-    for (; k >= 0; k = sPar[k]) {
+    while (k >= 0) {
+      const float4 xa = *reinterpret_cast<const float4*>(sXi + 8 * k), xb = *reinterpret_cast<const float4*>(sXi + 8 * k + 4);
+      const float old = row[k];
       while (key[0] == k) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) E[c] += es[0][c];
         pop();
       }
-      const float* xk = sXi + 6 * k;
-      row[k] -= xk[0] * E[0] + xk[1] * E[1] + xk[2] * E[2] + xk[3] * E[3] + xk[4] * E[4] + xk[5] * E[5];
+      row[k] = old - (xa.x * E[0] + xa.y * E[1] + xa.z * E[2] + xa.w * E[3] + xb.x * E[4] + xb.y * E[5]);
+      k = __float_as_int(xb.z);
     }
   }
 }
@@ -329,7 +333,6 @@ __device__ __forceinline__ void resid_jtj_impl(const Dev& d, BlockPos bp, int ph
   float* Js = reinterpret_cast<float*>(smem_raw);
   DQ* sHd = reinterpret_cast<DQ*>(Js + kBlock * ROW);
   float* sXi = reinterpret_cast<float*>(sHd + d.L);
-  int* sPar = reinterpret_cast<int*>(sXi + 6 * d.L);
   __shared__ int s_cnt[kMaxJtjGroup * (kBlock / 32)];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, G = d.jtj_group;
   const int NP = d.NP;
@@ -353,7 +356,7 @@ __device__ __forceinline__ void resid_jtj_impl(const Dev& d, BlockPos bp, int ph
     m[sub] = __ballot_sync(0xffffffffu, inA);
     if (lane == 0) s_cnt[sub * (kBlock / 32) + w] = __popc(m[sub]);
   }
-  load_link_tables(d, sHd, sXi, sPar);
+  load_link_tables(d, sHd, sXi);
   __syncthreads();
   int total = 0;
   for (int q = 0; q < G * (kBlock / 32); ++q) total += s_cnt[q];
@@ -392,11 +395,20 @@ __device__ __forceinline__ void resid_jtj_impl(const Dev& d, BlockPos bp, int ph
       rs.slot = tid;
       rs.base = bp.x * kBlock * G + c0;
       float r2;
-      jacobian_row(d, rs, phi_buf, Js, ROW, 16 * T, sHd, sXi, sPar, r2);
+      jacobian_row(d, rs, phi_buf, Js, ROW, 16 * T, sHd, sXi, r2);
     }
     __syncthreads();
-    if (h < S)
-      for (int s = h; s < rows; s += S) acc.add_row(Js + s * ROW, ty, tx);
+    if (h < S) {
+      // eight rows' loads ahead of their products (a row at a time waits for its loads: 62 cycles a row, not 25)
+      int s = h;
+#pragma unroll 1
+      for (; s + 7 * S < rows; s += 8 * S) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc.add_row(Js + (s + u * S) * ROW, ty, tx);
+      }
+#pragma unroll 1
+      for (; s < rows; s += S) acc.add_row(Js + s * ROW, ty, tx);
+    }
   }
   const int done = total;
   if (S > 1) {  // the groups' tiles, added into group 0's in group order
@@ -459,7 +471,6 @@ __device__ __forceinline__ void resid_jtj_tc_impl(const Dev& d, BlockPos bp, int
   float* Js = reinterpret_cast<float*>(smem_raw + TL::STAGE);
   DQ* sHd = reinterpret_cast<DQ*>(Js + kBlock * ROW);
   float* sXi = reinterpret_cast<float*>(sHd + d.L);
-  int* sPar = reinterpret_cast<int*>(sXi + 6 * d.L);
   __shared__ int s_warp[kBlock / 32];
   __shared__ float s_e[kBlock / 32];
   __shared__ uint64_t bar;
@@ -490,12 +501,12 @@ __device__ __forceinline__ void resid_jtj_tc_impl(const Dev& d, BlockPos bp, int
         tc::fence_mbar_init();
       }
       if (w == 0) tc::tmem_alloc(&tslot, tc::kTmemCols);
-      load_link_tables(d, sHd, sXi, sPar);
+      load_link_tables(d, sHd, sXi);
       taken = true;
     }
     __syncthreads();
     float r2;
-    jacobian_row(d, rs, phi_buf, Js, ROW, NP, sHd, sXi, sPar, r2);
+    jacobian_row(d, rs, phi_buf, Js, ROW, NP, sHd, sXi, r2);
     for (int o = 16; o > 0; o >>= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, o);
     if (lane == 0) s_e[w] = r2;
     tc::fence_before_sync();
@@ -686,12 +697,12 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_jtj(BatchGrid g, Dev 
 }
 
 static int jtj_smem_bytes(int T, int L) {
-  return kBlock * jtj_row_stride(T) * 4 + L * (int)sizeof(DQ) + 6 * L * 4 + L * 4;
+  return kBlock * jtj_row_stride(T) * 4 + L * (int)sizeof(DQ) + 8 * L * 4;
 }
 
 template <int PREC>
 static int jtj_tc_smem_bytes(int NB, int L) {
-  return tc::Tile<PREC, 8>::STAGE + kBlock * (16 * NB + 1) * 4 + L * (int)sizeof(DQ) + 6 * L * 4 + L * 4;
+  return tc::Tile<PREC, 8>::STAGE + kBlock * (16 * NB + 1) * 4 + L * (int)sizeof(DQ) + 8 * L * 4;
 }
 
 template <int PREC>
@@ -1849,13 +1860,26 @@ static void launch_resid_jtj_tc_b(const BatchGrid& g, int nblk, int max_np, int 
 }
 
 // gj[t - 1], nj[t - 1]: the blocks of the sessions whose [J r] tile width class is t = ceil(NP / 16)
-// (one launch per class, so a small skeleton does not pay for the largest one's tiles).
+// (one launch per class, so a small skeleton does not pay for the largest one's tiles).  A class of a few
+// sessions does not fill the chip, so the classes run beside each other where the caller has the streams for it
+// (eight uneven sessions, four classes of 86 to 492 blocks: one after the other they took 108 us).
 void launch_normal_equations_b(const BatchGrid* gj, const int* nj, const BatchGrid& gr, int nr, int max_links,
-                               int precision, int phi_buf, int slot, cudaStream_t st, int reduce_threads) {
+                               int precision, int phi_buf, int slot, cudaStream_t main, int reduce_threads,
+                               const ForkStreams* fork) {
+  int last = 0;
+  for (int T = 1; T <= 5; ++T)
+    if (nj[T - 1] > 0) last = T;
+  int sides = 0;
   for (int T = 1; T <= 5; ++T) {
     const BatchGrid& g = gj[T - 1];
     const int n = nj[T - 1];
     if (n == 0) continue;
+    cudaStream_t st = main;
+    if (fork && T != last) {
+      if (sides == 0) cudaEventRecord(fork->fork, main);
+      st = fork->side[sides];
+      cudaStreamWaitEvent(st, fork->fork, 0);
+    }
     if (precision == 1) {
       launch_resid_jtj_tc_b<1>(g, n, 16 * T, max_links, phi_buf, st);
     } else if (precision == 2) {
@@ -1870,8 +1894,10 @@ void launch_normal_equations_b(const BatchGrid* gj, const int* nj, const BatchGr
         default: k_resid_jtj<5><<<n, kBlock, sm, st>>>(g, Dev{}, phi_buf); break;
       }
     }
+    if (st != main) cudaEventRecord(fork->join[sides++], st);
   }
-  if (nr > 0) k_reduce_jtj<<<nr, reduce_threads, 0, st>>>(gr, Dev{}, slot);
+  for (int k = 0; k < sides; ++k) cudaStreamWaitEvent(main, fork->join[k], 0);
+  if (nr > 0) k_reduce_jtj<<<nr, reduce_threads, 0, main>>>(gr, Dev{}, slot);
 }
 
 void launch_lm_b(const BatchGrid& glm, int nlm, const BatchGrid& gv, int nv, int max_links, int phi_buf,

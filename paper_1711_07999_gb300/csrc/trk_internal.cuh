@@ -418,8 +418,14 @@ void launch_associate_b(const Dev* devs, int n_sessions, const AssocUnit* units,
                         int assoc_blocks, int tail_blocks, cudaStream_t st);
 void launch_gather_depth_b(const BatchGrid& g, int nblk, const float* const* srcs, AssocUnit* units, unsigned* ctl,
                            cudaStream_t st);
+// fork (may be null): streams on which the [J r] launches of the tile width classes run beside each other.
+struct ForkStreams {
+  cudaStream_t side[4] = {};
+  cudaEvent_t fork = nullptr, join[4] = {};
+};
 void launch_normal_equations_b(const BatchGrid* gj, const int* nj, const BatchGrid& gr, int nr, int max_links,
-                               int precision, int phi_buf, int slot, cudaStream_t st, int reduce_threads);
+                               int precision, int phi_buf, int slot, cudaStream_t st, int reduce_threads,
+                               const ForkStreams* fork = nullptr);
 void launch_lm_b(const BatchGrid& glm, int nlm, const BatchGrid& gv, int nv, int max_links, int phi_buf,
                  cudaStream_t st);
 int launch_shape_b(const BatchGrid& gv, int nv, int max_links, int sweeps, int solver, int phi_src, int slot,
