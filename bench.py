@@ -1131,7 +1131,7 @@ def run_ours(args, rank, world, local_rank):
             "uneven": uneven,
             "admission_serving": admission,
             "experiments": experiments,
-            "gpu_launches": (batched["schedule"]["groups"] * (info["kernels_per_frame"] + P + S) * args.steps
+            "gpu_launches": (batched["schedule"]["groups"] * info["kernels_per_frame"] * args.steps
                              if batched is not None else info["kernels_per_frame"] * args.steps),
             "roofline": roof,
             "stage_ms": {k: round(v, 5) for k, v in prof.items()},

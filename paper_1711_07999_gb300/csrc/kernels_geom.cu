@@ -435,6 +435,54 @@ __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, boo
 }
 
 
+// The same with four lanes per pixel (lane & 3): each takes two buckets of ring 1, the last one the pixel's own
+// too, and the (d^2, index) keys are combined by shuffles.  A pixel's thread walks its nine lists one
+// after the other, and a warp as long as its slowest lane at each of them; here that is two or three
+// steps.  It takes four times the warps, so it is for lists of units that leave most of them idle.
+__device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bool active) {
+  const Cam& c = d.cam;
+  const int lane = threadIdx.x & 31, sub = lane & 3;
+  const bool inimg = active && px < c.W && py < c.H;
+  const int k = py * c.W + px;
+  const float tau2 = c.tau * c.tau;
+  Best best{-1, 0.f, make_float3(0.f, 0.f, 0.f)};
+  float3 p = make_float3(0.f, 0.f, 0.f);
+  float dep = 0.f;
+  if (inimg) {
+    const float4 pp = d.ppos[k];
+    p = f3(pp);
+    dep = pp.w;
+    const int q[3] = {ring_bucket(px, py, 1, 2 * sub, c.W, c.H), ring_bucket(px, py, 1, 2 * sub + 1, c.W, c.H),
+                      sub == 3 ? k : -1};
+    scan_group<3, false>(d, q, p, tau2, best);
+  }
+  unsigned long long key = key_of(best.i, best.d2);
+  const unsigned long long mine = key;
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
+    key = other < key ? other : key;
+  }
+  bool open = false;
+  if (inimg) {
+    const float lb = dep * (1.0f + 0.499f) * c.kappa;
+    open = !(lb > c.tau || (key != ~0ull && lb * lb > __uint_as_float((unsigned)(key >> 32))) || c.R == 1);
+  }
+  const int nearest = key == ~0ull ? -1 : (int)(unsigned)(key & 0xffffffffu);
+  const unsigned om = __ballot_sync(0xffffffffu, open && sub == 0);
+  unsigned base = 0;
+  if (lane == 0 && om) base = atomicAdd(&d.qctl[0], __popc(om));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (sub == 0) {
+    if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int2(k, nearest);
+    else if (inimg) d.corr[k] = nearest;
+  }
+  const bool done = inimg && !open && nearest >= 0 && mine == key;  // the lane that holds the nearest
+  if (done) commit_pixel(d, best.i, p, best.v);
+  const unsigned m = __ballot_sync(0xffffffffu, done);
+  if (lane == 0 && m) atomicAdd(&d.stats[0], __popc(m));
+}
+
 constexpr int kTailWarps = 8;
 constexpr int kTailPerLane = 4;       // buckets a lane loads at once (one session: a warp per pixel)
 constexpr int kBatchTailLanes = 8;    // a batch's tail: lanes per queued pixel ...
@@ -546,28 +594,37 @@ __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const D
   const AssocUnit* list = single ? d0.units : units;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned nw = gridDim.x * (kBlock / 32);
-  if (single) {
-#pragma unroll 1
-    for (unsigned u = w * gridDim.x + blockIdx.x; u < n; u += nw) {
-      const int4 h = *reinterpret_cast<const int4*>(&list[u]);  // (session, x0, y0, pixels)
-      const int o = lane < h.w ? list[u].off[lane] : 0;
-      associate_impl(d0, h.y + (o & 15), h.z + (o >> 4), lane < h.w);
-    }
-    return;
-  }
+  // four lanes per pixel where that is at most two rounds of the grid's warps (the window search with R >= 1
+  // only); lane l of the warp then serves pixel 8 (part of the unit) + l / 4
+  const bool quad = 4 * n <= 2 * nw && (single ? d0.association == 0 && d0.cam.R > 0 : devs[0].association == 0);
+  const unsigned items = quad ? 4 * n : n;
   int cur = -1;
 #pragma unroll 1
-  for (unsigned u = w * gridDim.x + blockIdx.x; u < n; u += nw) {
-    const int4 h = *reinterpret_cast<const int4*>(&list[u]);
-    const int o = lane < h.w ? list[u].off[lane] : 0;
-    if (h.x != cur) {
+  for (unsigned it = w * gridDim.x + blockIdx.x; it < items; it += nw) {
+    const unsigned u = quad ? it >> 2 : it;
+    const int4 h = *reinterpret_cast<const int4*>(&list[u]);  // (session, x0, y0, pixels)
+    const int slot = quad ? 8 * (int)(it & 3) + (lane >> 2) : lane;
+    if (quad && 8 * (int)(it & 3) >= h.w) continue;
+    const int o = slot < h.w ? list[u].off[slot] : 0;
+    if (!single && h.x != cur) {
       __syncwarp();  // every lane is done with the previous descriptor
       const int* src = reinterpret_cast<const int*>(devs + h.x);
       for (int q = lane; q < (int)(sizeof(Dev) / 4); q += 32) reinterpret_cast<int*>(&sd[w])[q] = src[q];
       __syncwarp();
       cur = h.x;
     }
-    associate_impl(sd[w], h.y + (o & 15), h.z + (o >> 4), lane < h.w);
+    const int px = h.y + (o & 15), py = h.z + (o >> 4);
+    if (single) {
+      if (quad) associate4_impl(d0, px, py, slot < h.w);
+      else associate_impl(d0, px, py, slot < h.w);
+    } else {
+      if (quad && sd[w].cam.R > 0) {
+        associate4_impl(sd[w], px, py, slot < h.w);
+      } else if (!quad || (it & 3) == 0) {  // (a session without rings: the first item takes the whole unit)
+        const int o1 = lane < h.w ? list[u].off[lane] : 0;
+        associate_impl(sd[w], h.y + (o1 & 15), h.z + (o1 >> 4), lane < h.w);
+      }
+    }
   }
 }
 
@@ -589,7 +646,9 @@ __global__ void __launch_bounds__(32 * kTailWarps) k_associate_tail(Dev d) {
   if (gl == 0 && done) atomicAdd(&d.stats[0], done);
 }
 
-// A batch: prefix[s] = queued pixels of the sessions before s (one block; at most 1024 x 4 sessions).
+constexpr int kInBlockPrefix = 32 * kTailWarps;  // sessions whose prefix the tail's blocks form themselves
+
+// A larger batch: prefix[s] = queued pixels of the sessions before s (one block; at most 1024 x 4 sessions).
 __global__ void __launch_bounds__(1024) k_tail_prefix(const Dev* devs, int n_sessions, unsigned* prefix) {
   __shared__ unsigned part[1024];
   const int t = threadIdx.x;
@@ -620,10 +679,31 @@ __global__ void __launch_bounds__(1024) k_tail_prefix(const Dev* devs, int n_ses
 // the rest from one counter; an entry's session is found in the prefix and its descriptor read through
 // the cache.
 __global__ void __launch_bounds__(32 * kTailWarps, kTailBlocksPerSM) k_associate_tail_batch(const Dev* devs, int n_sessions,
-                                                                          const unsigned* prefix, unsigned* ctl) {
+                                                                          const unsigned* global_prefix, unsigned* ctl) {
   constexpr int GL = kBatchTailLanes;
   const int lane = threadIdx.x & 31, gl = lane % GL, gbase = lane - gl;
   const unsigned gmask = ((1u << GL) - 1u) << gbase;
+  // up to kInBlockPrefix sessions every block forms the prefix itself (a launch less); more: k_tail_prefix
+  __shared__ unsigned s_prefix[kInBlockPrefix + 1], s_sum[kTailWarps];
+  const unsigned* prefix = global_prefix;
+  if (n_sessions <= kInBlockPrefix) {
+    static_assert(kInBlockPrefix == 32 * kTailWarps, "a session per thread");
+    const int t = threadIdx.x, wp = t >> 5;
+    const unsigned v = t < n_sessions ? *(volatile unsigned*)&devs[t].qctl[0] : 0u;
+    unsigned sum = v;  // inclusive scan over the warp, then the warps' totals before it
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned x = __shfl_up_sync(0xffffffffu, sum, o);
+      sum += lane >= o ? x : 0u;
+    }
+    if (lane == 31) s_sum[wp] = sum;
+    __syncthreads();
+    for (int q = 0; q < wp; ++q) sum += s_sum[q];
+    s_prefix[t + 1] = sum;
+    if (t == 0) s_prefix[0] = 0;
+    __syncthreads();
+    prefix = s_prefix;
+  }
   const unsigned total = prefix[n_sessions];
   const unsigned groups = gridDim.x * (blockDim.x / GL);  // group g takes entry g first, then the counter's
   for (unsigned item = (blockIdx.x * blockDim.x + threadIdx.x) / GL; item < total;) {
@@ -716,7 +796,7 @@ void launch_visibility_b(const BatchGrid& g, int nblk, cudaStream_t st) {
 void launch_associate_b(const Dev* devs, int n_sessions, const AssocUnit* tiles, unsigned* ctl, unsigned* prefix,
                         int assoc_blocks, int tail_blocks, cudaStream_t st) {
   k_associate<<<assoc_blocks, kBlock, 0, st>>>(devs, tiles, ctl, Dev{});
-  k_tail_prefix<<<1, 1024, 0, st>>>(devs, n_sessions, prefix);
+  if (n_sessions > kInBlockPrefix) k_tail_prefix<<<1, 1024, 0, st>>>(devs, n_sessions, prefix);
   k_associate_tail_batch<<<tail_blocks, 32 * kTailWarps, 0, st>>>(devs, n_sessions, prefix, ctl);
 }
 

@@ -1418,6 +1418,8 @@ __global__ void __launch_bounds__(kBlock) k_lm_eval(BatchGrid g, Dev d0) {
     lm_eval_impl<c0, c1>(d0, grid_pos());
     return;
   }
+  // the second pass mostly has nothing to do: looked up before the descriptor is staged
+  if (c0 > 0 && g.devs[g.map[blockIdx.x].x].lm_trials[7] != kPending) return;
   __shared__ Dev sd;
   lm_eval_impl<c0, c1>(sd, batch_block(g, sd));
 }
