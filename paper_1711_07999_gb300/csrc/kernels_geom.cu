@@ -594,9 +594,11 @@ __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const D
   const AssocUnit* list = single ? d0.units : units;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned nw = gridDim.x * (kBlock / 32);
-  // four lanes per pixel where that is at most two rounds of the grid's warps (the window search with R >= 1
+  // four lanes per pixel where the units do not fill the grid's warps even once, so that the launch lasts as long as
+  // a unit (3,500 units of uneven sessions on 4,864 warps: 69 us a lane per pixel, 41 four; 9,600 units of
+  // sixteen equal ones: 34 against 40) (the window search with R >= 1
   // only); lane l of the warp then serves pixel 8 (part of the unit) + l / 4
-  const bool quad = 4 * n <= 2 * nw && (single ? d0.association == 0 && d0.cam.R > 0 : devs[0].association == 0);
+  const bool quad = n <= nw && (single ? d0.association == 0 && d0.cam.R > 0 : devs[0].association == 0);
   const unsigned items = quad ? 4 * n : n;
   int cur = -1;
 #pragma unroll 1

@@ -1463,6 +1463,19 @@ __device__ __forceinline__ float3 solve3_damped(float3 g, float cdiag, float lw,
                      (c02 * rhs.x + c12 * rhs.y + c22 * rhs.z) * id);
 }
 
+// Sum of v[0 .. kBlock) as a binary tree over the threads (v[t] += v[t + h], h = 128, .., 1), in thread 0; the
+// last five levels by shuffles.  The caller has synchronised after writing v.
+__device__ __forceinline__ double block_tree(double* v) {
+  for (int h = kBlock / 2; h >= 32; h >>= 1) {
+    if (threadIdx.x < h) v[threadIdx.x] += v[threadIdx.x + h];
+    __syncthreads();
+  }
+  double x = threadIdx.x < 32 ? v[threadIdx.x] : 0.0;
+  if (threadIdx.x < 32)
+    for (int h = 16; h > 0; h >>= 1) x += __shfl_down_sync(0xffffffffu, x, h);
+  return x;
+}
+
 __device__ __forceinline__ void block_energy_to_slot(const Dev& d, BlockPos bp, float e, int slot, int ticket) {
   __shared__ double sw[kBlock];
   __shared__ bool last;
@@ -1483,12 +1496,9 @@ __device__ __forceinline__ void block_energy_to_slot(const Dev& d, BlockPos bp, 
   for (int b = threadIdx.x; b < bp.gx; b += kBlock) s += __ldcg(d.epart + (size_t)b * 8);
   sw[threadIdx.x] = s;
   __syncthreads();
-  for (int h = kBlock / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) sw[threadIdx.x] += sw[threadIdx.x + h];
-    __syncthreads();
-  }
+  const double total = block_tree(sw);
   if (threadIdx.x == 0) {
-    if (slot >= 0) d.energy[slot] = sw[0];
+    if (slot >= 0) d.energy[slot] = total;
     d.counter[ticket] = 0;
   }
 }
@@ -1646,13 +1656,38 @@ __device__ __forceinline__ bool block_total(const Dev& d, BlockPos bp, double v,
   for (int b = threadIdx.x; b < bp.gx; b += kBlock) s += __ldcg(d.epart + (size_t)b * 8 + slot);
   red[threadIdx.x] = s;
   __syncthreads();
-  for (int h = kBlock / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-    __syncthreads();
-  }
-  total = red[0];
+  total = block_tree(red);
   if (threadIdx.x == 0) d.counter[ticket] = 0;
   return true;
+}
+
+// a.b in FP64 (products of FP32 numbers are exact there), whole warps; the conversions without the FP64 pipe.
+__device__ __forceinline__ double dot3_fp64(float3 a, float3 b) {
+  bool other = false;
+  double ax = widen(a.x, other), ay = widen(a.y, other), az = widen(a.z, other);
+  double bx = widen(b.x, other), by = widen(b.y, other), bz = widen(b.z, other);
+  if (__any_sync(0xffffffffu, other)) {
+    ax = (double)a.x, ay = (double)a.y, az = (double)a.z;
+    bx = (double)b.x, by = (double)b.y, bz = (double)b.z;
+  }
+  return ax * bx + ay * by + az * bz;
+}
+
+// Sums f(neighbour) over the neighbourhood edges [a0, a1) of a vertex in order, eight loads in flight.
+template <typename Load, typename Add>
+__device__ __forceinline__ void for_neighbours(const Dev& d, int a0, int a1, Load load, Add add) {
+  for (int t = a0; t < a1; t += 8) {
+    int j[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) j[u] = t + u < a1 ? d.adj[t + u] : -1;
+    float3 q[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (j[u] >= 0) q[u] = load(j[u]);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (j[u] >= 0) add(q[u]);
+  }
 }
 
 // B_i = M_i + lambda_w diag(M_i), M_i = g g^T + c I (g = 0 outside A): B_i p and B_i^-1 p.
@@ -1674,7 +1709,7 @@ __device__ __forceinline__ void cg_init_impl(const Dev& d, BlockPos bp, int src,
     __syncthreads();
   }
   float e = 0.f;
-  double rz = 0.0;
+  float3 rr = make_float3(0.f, 0.f, 0.f), z = rr;
   int inA_count = 0;
   if (i < d.V) {
     const float4* phi = d.phi[src];
@@ -1699,22 +1734,20 @@ __device__ __forceinline__ void cg_init_impl(const Dev& d, BlockPos bp, int src,
     }
     float3 sd = make_float3(0.f, 0.f, 0.f);
     const int a0 = d.adj_off[i], a1 = d.adj_off[i + 1];
-    for (int t = a0; t < a1; ++t) {
-      const float3 q = f3(phi[d.adj[t]]);
-      sd.x += pi.x - q.x; sd.y += pi.y - q.y; sd.z += pi.z - q.z;
-    }
-    const float3 rr = make_float3(-(g.x * r + d.lambda_phi * pi.x + d.lambda_N * sd.x),
-                                  -(g.y * r + d.lambda_phi * pi.y + d.lambda_N * sd.y),
-                                  -(g.z * r + d.lambda_phi * pi.z + d.lambda_N * sd.z));
-    const float3 z = solve3_damped(g, d.lambda_phi + d.lambda_N * (float)(a1 - a0), d.lambda_w, rr);
+    for_neighbours(d, a0, a1, [&](int j) { return f3(phi[j]); },
+                   [&](float3 q) { sd.x += pi.x - q.x; sd.y += pi.y - q.y; sd.z += pi.z - q.z; });
+    rr = make_float3(-(g.x * r + d.lambda_phi * pi.x + d.lambda_N * sd.x),
+                     -(g.y * r + d.lambda_phi * pi.y + d.lambda_N * sd.y),
+                     -(g.z * r + d.lambda_phi * pi.z + d.lambda_N * sd.z));
+    z = solve3_damped(g, d.lambda_phi + d.lambda_N * (float)(a1 - a0), d.lambda_w, rr);
     d.rg[i] = make_float4(g.x, g.y, g.z, r);
     d.phi0[i] = p4;
     d.cg_x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     d.cg_r[i] = make_float4(rr.x, rr.y, rr.z, 0.f);
     d.cg_z[i] = make_float4(z.x, z.y, z.z, 0.f);
-    d.cg_p[i] = make_float4(z.x, z.y, z.z, 0.f);
-    rz = (double)rr.x * z.x + (double)rr.y * z.y + (double)rr.z * z.z;
+    d.cg_p[0][i] = make_float4(z.x, z.y, z.z, 0.f);
   }
+  const double rz = dot3_fp64(rr, z);
   const unsigned m = __ballot_sync(0xffffffffu, inA_count != 0);
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(&d.stats[1], __popc(m));
   double tot;
@@ -1725,22 +1758,31 @@ __device__ __forceinline__ void cg_init_impl(const Dev& d, BlockPos bp, int src,
   block_energy_to_slot(d, bp, e, slot, 1);
 }
 
-// Ap = (B - lambda_N Adj) p; alpha = r.z / p.Ap (0 and stop on a breakdown).
-__device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp) {
+// Iteration k > 0: p = z + beta p first (the neighbours' too, each formed from its z and old p, so that the
+// direction needs no pass of its own; p is written to the other buffer).  Ap = (B - lambda_N Adj) p;
+// alpha = r.z / p.Ap (0 and stop on a breakdown).
+__device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp, int k) {
   const int i = bp.x * kBlock + threadIdx.x;
-  double pap = 0.0;
+  float3 p = make_float3(0.f, 0.f, 0.f), ap = p;
   if (i < d.V) {
+    const float beta = (float)d.cg[2];
+    const float4* old = d.cg_p[(k - 1) & 1];
+    auto direction = [&](int j) {
+      if (k == 0) return f3(d.cg_p[0][j]);
+      const float3 z = f3(d.cg_z[j]), q = f3(old[j]);
+      return make_float3(z.x + beta * q.x, z.y + beta * q.y, z.z + beta * q.z);
+    };
     const float4 rg = d.rg[i];
-    const float3 p = f3(d.cg_p[i]);
+    p = direction(i);
+    if (k > 0) d.cg_p[k & 1][i] = make_float4(p.x, p.y, p.z, 0.f);
     const int a0 = d.adj_off[i], a1 = d.adj_off[i + 1];
-    float3 ap = block_apply(f3(rg), d.lambda_phi + d.lambda_N * (float)(a1 - a0), d.lambda_w, p);
-    for (int t = a0; t < a1; ++t) {
-      const float3 q = f3(d.cg_p[d.adj[t]]);
+    ap = block_apply(f3(rg), d.lambda_phi + d.lambda_N * (float)(a1 - a0), d.lambda_w, p);
+    for_neighbours(d, a0, a1, direction, [&](float3 q) {
       ap.x -= d.lambda_N * q.x; ap.y -= d.lambda_N * q.y; ap.z -= d.lambda_N * q.z;
-    }
+    });
     d.cg_ap[i] = make_float4(ap.x, ap.y, ap.z, 0.f);
-    pap = (double)p.x * ap.x + (double)p.y * ap.y + (double)p.z * ap.z;
   }
+  const double pap = dot3_fp64(p, ap);
   double tot;
   if (block_total(d, bp, pap, 2, 3, tot) && threadIdx.x == 0) {
     const bool go = d.cg[3] == 0.0 && tot > 0.0;
@@ -1749,24 +1791,30 @@ __device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp) {
   }
 }
 
-// x += alpha p, r -= alpha Ap, z = B^-1 r; beta = r.z_new / r.z.
-__device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp) {
+// x += alpha p, r -= alpha Ap, z = B^-1 r; beta = r.z_new / r.z.  The last iteration (out >= 0): phi[out] =
+// phi[1 - out] + x.
+__device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int k, int out) {
   const int i = bp.x * kBlock + threadIdx.x;
-  const float alpha = (float)d.cg[1];
-  double rz = 0.0;
+  float3 r = make_float3(0.f, 0.f, 0.f), z = r;
   if (i < d.V) {
+    const float alpha = (float)d.cg[1];
     const float4 rg = d.rg[i];
-    const float3 p = f3(d.cg_p[i]), ap = f3(d.cg_ap[i]);
-    float3 x = f3(d.cg_x[i]), r = f3(d.cg_r[i]);
+    const float3 p = f3(d.cg_p[k & 1][i]), ap = f3(d.cg_ap[i]);
+    float3 x = f3(d.cg_x[i]);
+    r = f3(d.cg_r[i]);
     x.x += alpha * p.x; x.y += alpha * p.y; x.z += alpha * p.z;
     r.x -= alpha * ap.x; r.y -= alpha * ap.y; r.z -= alpha * ap.z;
     const int deg = d.adj_off[i + 1] - d.adj_off[i];
-    const float3 z = solve3_damped(f3(rg), d.lambda_phi + d.lambda_N * (float)deg, d.lambda_w, r);
+    z = solve3_damped(f3(rg), d.lambda_phi + d.lambda_N * (float)deg, d.lambda_w, r);
     d.cg_x[i] = make_float4(x.x, x.y, x.z, 0.f);
     d.cg_r[i] = make_float4(r.x, r.y, r.z, 0.f);
     d.cg_z[i] = make_float4(z.x, z.y, z.z, 0.f);
-    rz = (double)r.x * z.x + (double)r.y * z.y + (double)r.z * z.z;
+    if (out >= 0) {
+      const float4 f = d.phi[1 - out][i];
+      d.phi[out][i] = make_float4(f.x + x.x, f.y + x.y, f.z + x.z, 0.f);
+    }
   }
+  const double rz = dot3_fp64(r, z);
   double tot;
   if (block_total(d, bp, rz, 1, 2, tot) && threadIdx.x == 0) {
     const bool go = d.cg[3] == 0.0 && d.cg[0] > 0.0;
@@ -1774,23 +1822,6 @@ __device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp) {
     d.cg[0] = tot;
     if (!(tot > 0.0)) d.cg[3] = 1.0;
   }
-}
-
-// p = z + beta p.
-__device__ __forceinline__ void cg_dir_impl(const Dev& d, BlockPos bp) {
-  const int i = bp.x * kBlock + threadIdx.x;
-  if (i >= d.V) return;
-  const float beta = (float)d.cg[2];
-  const float3 z = f3(d.cg_z[i]), p = f3(d.cg_p[i]);
-  d.cg_p[i] = make_float4(z.x + beta * p.x, z.y + beta * p.y, z.z + beta * p.z, 0.f);
-}
-
-// phi[1 - src] = phi[src] + x.
-__device__ __forceinline__ void cg_finish_impl(const Dev& d, BlockPos bp, int src) {
-  const int i = bp.x * kBlock + threadIdx.x;
-  if (i >= d.V) return;
-  const float4 p = d.phi[src][i], x = d.cg_x[i];
-  d.phi[1 - src][i] = make_float4(p.x + x.x, p.y + x.y, p.z + x.z, 0.f);
 }
 
 #define TRK_CG_KERNEL(name, impl, ...)                                                     \
@@ -1804,19 +1835,13 @@ __device__ __forceinline__ void cg_finish_impl(const Dev& d, BlockPos bp, int sr
   }
 #define ARGS_k_cg_init , int src, int slot
 #define CALL_k_cg_init , src, slot
-#define ARGS_k_cg_apply
-#define CALL_k_cg_apply
-#define ARGS_k_cg_update
-#define CALL_k_cg_update
-#define ARGS_k_cg_dir
-#define CALL_k_cg_dir
-#define ARGS_k_cg_finish , int src
-#define CALL_k_cg_finish , src
+#define ARGS_k_cg_apply , int k
+#define CALL_k_cg_apply , k
+#define ARGS_k_cg_update , int k, int out
+#define CALL_k_cg_update , k, out
 TRK_CG_KERNEL(k_cg_init, cg_init_impl)
 TRK_CG_KERNEL(k_cg_apply, cg_apply_impl)
 TRK_CG_KERNEL(k_cg_update, cg_update_impl)
-TRK_CG_KERNEL(k_cg_dir, cg_dir_impl)
-TRK_CG_KERNEL(k_cg_finish, cg_finish_impl)
 
 // The whole coupled step (g, n: the block table and its size for a batch; kSingle and nblk_v alone).
 static void launch_shape_pcg(const BatchGrid& g, int n, const Dev& d0, int max_links, int iters, int src, int slot,
@@ -1824,11 +1849,9 @@ static void launch_shape_pcg(const BatchGrid& g, int n, const Dev& d0, int max_l
   if (n <= 0) return;
   k_cg_init<<<n, kBlock, max_links * sizeof(DQ), st>>>(g, d0, src, slot);
   for (int k = 0; k < iters; ++k) {
-    k_cg_apply<<<n, kBlock, 0, st>>>(g, d0);
-    k_cg_update<<<n, kBlock, 0, st>>>(g, d0);
-    if (k + 1 < iters) k_cg_dir<<<n, kBlock, 0, st>>>(g, d0);
+    k_cg_apply<<<n, kBlock, 0, st>>>(g, d0, k);
+    k_cg_update<<<n, kBlock, 0, st>>>(g, d0, k, k + 1 < iters ? -1 : 1 - src);
   }
-  k_cg_finish<<<n, kBlock, 0, st>>>(g, d0, src);
 }
 
 // Returns the buffer that holds Phi after the step.

@@ -540,10 +540,10 @@ void carve_all(trk_session* s) {
   carve(s, &d.units, (size_t)kUnitsPerTile * ((d.cam.W + 15) / 16) * ((d.cam.H + 15) / 16));
   carve(s, &d.acc, V); carve(s, &d.vispix, V); carve(s, &d.rg, V); carve(s, &d.phi0, V);
   carve(s, &dadj_off, V + 1); carve(s, &dadj, s->hm.adj.size());
-  d.cg_x = d.cg_r = d.cg_z = d.cg_p = d.cg_ap = nullptr;
+  d.cg_x = d.cg_r = d.cg_z = d.cg_p[0] = d.cg_p[1] = d.cg_ap = nullptr;
   if (prm.shape_solver == 1) {
     carve(s, &d.cg_x, V); carve(s, &d.cg_r, V); carve(s, &d.cg_z, V);
-    carve(s, &d.cg_p, V); carve(s, &d.cg_ap, V);
+    carve(s, &d.cg_p[0], V); carve(s, &d.cg_p[1], V); carve(s, &d.cg_ap, V);
   }
   carve(s, &d.cg, 4);
   carve(s, &ddepth, npx);
@@ -1232,7 +1232,7 @@ trk_status trk_get_info(trk_session* s, trk_info* out) {
   out->width = d.cam.W;
   out->height = d.cam.H;
   const int per_assoc = (d.F > 0 ? 5 : 4);  // skin, raster, visibility, associate (2 kernels)
-  const int shape_k = s->prm.shape_solver == 1 ? 3 * s->prm.shape_sweeps + 1 : s->prm.shape_sweeps;
+  const int shape_k = s->prm.shape_solver == 1 ? 2 * s->prm.shape_sweeps + 1 : s->prm.shape_sweeps;
   out->kernels_per_frame = 1 + s->prm.pose_iters * (per_assoc + 5) + s->prm.shape_iters * (per_assoc + shape_k);
   out->device_bytes = s->device_bytes;
   out->jtj_group = s->d.jtj_group;

@@ -388,7 +388,7 @@ struct Dev {
   int association;        // 0 window search, 1 nearest corner of the rasterised triangle
   const int* adj_off;     // [V + 1] neighbourhood edges of each vertex in both directions (CSR) ...
   const int* adj;         // ... sorted by vertex index
-  float4 *cg_x, *cg_r, *cg_z, *cg_p, *cg_ap;  // [V] PCG vectors
+  float4 *cg_x, *cg_r, *cg_z, *cg_p[2], *cg_ap;  // [V] PCG vectors (the direction of iteration k in cg_p[k & 1])
   double* cg;             // [4] rz, alpha, beta, stopped
 };
 
