@@ -337,17 +337,46 @@ trk_status batch_create(trk_session* const* sessions, int n_sessions, int assoc_
 // written straight from / into host-mapped pinned memory (zero copy over the chip-to-chip link), so a
 // step costs its launches, one small upload and no per-session copies.
 
+// Vertex block vb of a session's results.  The offsets go out as [V][3] through shared memory, so that the host
+// memory behind the chip-to-chip link is written in 16-byte pieces and the host only copies them (it used
+// to receive 16 bytes per vertex and pick the three floats in a loop: 200k vertices, 1.6x the time of a frame's
+// result).
+__device__ __forceinline__ void results_impl(const Dev& d, const ResultDst& o, int vb) {
+  __shared__ __align__(16) float s_phi[3 * 256];
+  const int t = threadIdx.x, n = min(256, d.V - 256 * vb);  // vertices of this block
+  if (o.phi) {
+    if (t < n) {
+      const float4 p = d.phi[0][256 * vb + t];
+      s_phi[3 * t] = p.x;
+      s_phi[3 * t + 1] = p.y;
+      s_phi[3 * t + 2] = p.z;
+    }
+    __syncthreads();
+    float* out = o.phi + (size_t)768 * vb;
+    for (int q = 4 * t; q < 3 * n; q += 4 * 256) {
+      if (q + 3 < 3 * n) {
+        *reinterpret_cast<float4*>(out + q) = *reinterpret_cast<const float4*>(s_phi + q);
+      } else {
+        for (int c = q; c < 3 * n; ++c) out[c] = s_phi[c];
+      }
+    }
+  }
+  if (vb == 0) {
+    for (int k = t; k < d.L; k += blockDim.x) o.theta[k] = d.theta[k];
+    for (int k = t; k < d.pose_iters + d.shape_iters; k += blockDim.x) o.energy[k] = d.energy[k];
+    if (t < 4) o.stats[t] = d.stats[t];
+  }
+}
+
 __global__ void __launch_bounds__(256) k_results_b(BatchGrid g, const ResultDst* __restrict__ dst) {
   const int4 m = g.map[blockIdx.x];
-  const Dev& d = g.devs[m.x];
-  const ResultDst o = dst[m.x];
-  const int i = m.y * 256 + threadIdx.x;
-  if (i < d.V) o.phi[i] = d.phi[0][i];
-  if (m.y == 0) {
-    for (int t = threadIdx.x; t < d.L; t += blockDim.x) o.theta[t] = d.theta[t];
-    for (int t = threadIdx.x; t < d.pose_iters + d.shape_iters; t += blockDim.x) o.energy[t] = d.energy[t];
-    if (threadIdx.x < 4) o.stats[threadIdx.x] = d.stats[threadIdx.x];
-  }
+  results_impl(g.devs[m.x], dst[m.x], m.y);
+}
+
+__global__ void __launch_bounds__(256) k_results(Dev d, ResultDst dst) { results_impl(d, dst, blockIdx.x); }
+
+void launch_results(const Dev& d, const ResultDst& dst, cudaStream_t st) {
+  k_results<<<dst.phi ? std::max((d.V + 255) / 256, 1) : 1, 256, 0, st>>>(d, dst);
 }
 
 struct BatchStep {

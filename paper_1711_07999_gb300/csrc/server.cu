@@ -38,7 +38,7 @@ trk_status session_evict(trk_session* s);
 trk_status session_restore(trk_session* s);
 const trk_params& session_params(const trk_session* s);
 trk_status session_enqueue_frame(trk_session* s, const float* host_depth, cudaStream_t* stream_out);
-trk_status session_enqueue_results(trk_session* s, double* theta, float* phi4, double* energy, int* stats);
+trk_status session_enqueue_results(trk_session* s, const ResultDst& dst);
 void session_result_sizes(const trk_session* s, int* n_links, int* n_verts, int* n_energy);
 void session_forget_stream(trk_session* s, cudaStream_t st);
 }  // namespace trk
@@ -87,7 +87,7 @@ struct Staging {
   double* theta = nullptr;   // [L]
   double* energy = nullptr;  // [ne]
   int* stats = nullptr;      // [4]
-  float4* phi = nullptr;     // [V]
+  float* phi = nullptr;      // [V][3]
   const float* depth_dev = nullptr;  // device addresses of the same memory
   trk::ResultDst dst{};
 };
@@ -167,7 +167,7 @@ Staging* new_staging(size_t npx, int L, int V, int ne) {
   Staging* b = new Staging();
   const size_t o_th = up16(sizeof(float) * npx), o_en = o_th + up16(sizeof(double) * L),
                o_st = o_en + up16(sizeof(double) * std::max(ne, 1)), o_phi = o_st + 16,
-               total = o_phi + sizeof(float4) * std::max(V, 1);
+               total = o_phi + 3 * sizeof(float) * std::max(V, 1);
   if (cudaHostAlloc(&b->block, total, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
     delete b;
     return nullptr;
@@ -186,12 +186,12 @@ Staging* new_staging(size_t npx, int L, int V, int ne) {
   b->theta = reinterpret_cast<double*>(h + o_th);
   b->energy = reinterpret_cast<double*>(h + o_en);
   b->stats = reinterpret_cast<int*>(h + o_st);
-  b->phi = reinterpret_cast<float4*>(h + o_phi);
+  b->phi = reinterpret_cast<float*>(h + o_phi);
   b->depth_dev = reinterpret_cast<const float*>(dev);
   b->dst.theta = reinterpret_cast<double*>(dev + o_th);
   b->dst.energy = reinterpret_cast<double*>(dev + o_en);
   b->dst.stats = reinterpret_cast<int*>(dev + o_st);
-  b->dst.phi = reinterpret_cast<float4*>(dev + o_phi);
+  b->dst.phi = reinterpret_cast<float*>(dev + o_phi);
   return b;
 }
 
@@ -269,7 +269,7 @@ void launch_session(trk_server* sv, trk_session* s, SessionSlot& sl) {
   st->reqs.push_back(r);
   trk_status e = trk::session_enqueue_frame(s, r->b->depth, &st->st);
   if (e == TRK_OK)
-    e = trk::session_enqueue_results(s, r->b->theta, reinterpret_cast<float*>(r->b->phi), r->b->energy, r->b->stats);
+    e = trk::session_enqueue_results(s, r->b->dst);
   if (e == TRK_OK && cudaLaunchHostFunc(st->st, on_step_done, st) != cudaSuccess) e = TRK_ERR_CUDA;
   if (e != TRK_OK) {
     fail_requests(sv, st->reqs, e);
@@ -608,12 +608,7 @@ trk_status trk_server_wait(trk_server* sv, uint64_t ticket, int64_t timeout_us, 
     trk::session_result_sizes(r->s, &L, &V, &ne);
     if (out->theta) std::memcpy(out->theta, b->theta, sizeof(double) * L);
     if (out->energy) std::memcpy(out->energy, b->energy, sizeof(double) * ne);
-    if (out->offsets)
-      for (int i = 0; i < V; ++i) {
-        out->offsets[3 * i] = b->phi[i].x;
-        out->offsets[3 * i + 1] = b->phi[i].y;
-        out->offsets[3 * i + 2] = b->phi[i].z;
-      }
+    if (out->offsets) std::memcpy(out->offsets, b->phi, 3 * sizeof(float) * V);
     out->n_assoc_px = b->stats[0];
     out->n_assoc_verts = b->stats[1];
   }

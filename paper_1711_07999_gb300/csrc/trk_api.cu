@@ -265,7 +265,7 @@ struct trk_session {
   double ev_lam = 0.0;
   std::vector<float4> ev_phi;
   double* h_pinned = nullptr;  // pinned staging for results
-  float4* h_phi = nullptr;     // pinned staging for the offsets of a result [V]
+  float* h_phi = nullptr;      // pinned staging for the offsets of a result [V][3]
   float* d_render = nullptr;
 };
 
@@ -406,11 +406,14 @@ trk_status fetch_result(trk_session* s, cudaStream_t st, trk_result* out) {
   const Dev& d = s->d;
   const int ne = s->prm.pose_iters + s->prm.shape_iters;
   double* h = s->h_pinned;  // [L] theta, [ne] energy, [1] stats
-  CK(cudaMemcpyAsync(h, d.theta, sizeof(double) * d.L, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h + d.L, d.energy, sizeof(double) * ne, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h + d.L + ne, d.stats, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
-  const float4* phi = s->h_phi;
-  if (out->offsets) CK(cudaMemcpyAsync(s->h_phi, d.phi[0], sizeof(float4) * d.V, cudaMemcpyDeviceToHost, st));
+  // one kernel writes them straight into the pinned memory (a copy each cost more than the copying)
+  ResultDst dst{};
+  dst.theta = h;
+  dst.energy = h + d.L;
+  dst.stats = reinterpret_cast<int*>(h + d.L + ne);
+  dst.phi = out->offsets ? s->h_phi : nullptr;
+  launch_results(d, dst, st);
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
   if (out->theta) std::memcpy(out->theta, h, sizeof(double) * d.L);
   if (out->energy) std::memcpy(out->energy, h + d.L, sizeof(double) * ne);
@@ -419,12 +422,7 @@ trk_status fetch_result(trk_session* s, cudaStream_t st, trk_result* out) {
   out->n_assoc_px = stats[0];
   out->n_assoc_verts = stats[1];
   if (stats[3]) return fail(TRK_ERR_TIMEOUT, "a tensor-core completion wait ran out; results are not valid");
-  if (out->offsets)
-    for (int i = 0; i < d.V; ++i) {
-      out->offsets[3 * i] = phi[i].x;
-      out->offsets[3 * i + 1] = phi[i].y;
-      out->offsets[3 * i + 2] = phi[i].z;
-    }
+  if (out->offsets) std::memcpy(out->offsets, s->h_phi, 3 * sizeof(float) * d.V);
   return TRK_OK;
 }
 
@@ -469,14 +467,10 @@ trk_status session_enqueue_frame(trk_session* s, const float* host_depth, cudaSt
   *stream_out = s->stream;
   return TRK_OK;
 }
-// D2H of the frame's results into (pinned) host buffers, on the session's stream
-trk_status session_enqueue_results(trk_session* s, double* theta, float* phi4, double* energy, int* stats) {
-  const Dev& d = s->d;
-  const int ne = s->prm.pose_iters + s->prm.shape_iters;
-  CK(cudaMemcpyAsync(theta, d.theta, sizeof(double) * d.L, cudaMemcpyDeviceToHost, s->stream));
-  CK(cudaMemcpyAsync(phi4, d.phi[0], sizeof(float4) * d.V, cudaMemcpyDeviceToHost, s->stream));
-  if (ne > 0) CK(cudaMemcpyAsync(energy, d.energy, sizeof(double) * ne, cudaMemcpyDeviceToHost, s->stream));
-  CK(cudaMemcpyAsync(stats, d.stats, sizeof(int) * 4, cudaMemcpyDeviceToHost, s->stream));
+// The frame's results into (pinned) host buffers, on the session's stream
+trk_status session_enqueue_results(trk_session* s, const ResultDst& dst) {
+  launch_results(s->d, dst, s->stream);
+  CK(cudaGetLastError());
   return TRK_OK;
 }
 }  // namespace trk
@@ -868,7 +862,7 @@ trk_status create_session(const trk_mesh* mesh, const trk_skeleton* sk, const tr
     s->device_bytes = (std::max<size_t>(s->carved, 1) + g - 1) / g * g;
   }
   CK(cudaMallocHost(&s->h_pinned, sizeof(double) * (L + prm->pose_iters + prm->shape_iters + 4)));
-  CK(cudaMallocHost(&s->h_phi, sizeof(float4) * std::max(V, 1)));
+  CK(cudaMallocHost(&s->h_phi, 3 * sizeof(float) * std::max(V, 1)));
   // the state of trk_set_pose(Theta = 0, Phi = 0)
   s->ev_theta.assign(L, 0.0);
   s->ev_lam = prm->lambda_k0;

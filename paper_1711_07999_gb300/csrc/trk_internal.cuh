@@ -448,10 +448,12 @@ struct BatchGrid {
 // Where a batched step writes one session's results (device-accessible, e.g. host-mapped pinned memory).
 struct ResultDst {
   double* theta;   // [L]
-  float4* phi;     // [V] (x, y, z, 0)
+  float* phi;      // [V][3], 16-byte aligned (null: not wanted)
   double* energy;  // [pose_iters + shape_iters]
   int* stats;      // [4]
 };
+// One session's results into dst (device-accessible; pinned host memory is).
+void launch_results(const Dev& d, const ResultDst& dst, cudaStream_t st);
 struct BatchStep;
 // device bytes one session adds to a step's buffer (a buffer holds at most twice its step's sum, rounded
 // up to the allocation granularity)
