@@ -233,12 +233,11 @@ void launch_visibility(const Dev& d, cudaStream_t st) {
 // that angle into a distance from p), so the search stops once that bound exceeds the best distance
 // or tau: the result is the same argmin as the exhaustive window search.
 //
-// k_associate: rings 0..kRingsPerThread by the pixel's own thread, four buckets' heads and first records
-// loaded together.  Pixels still open after that (the bound of ring 1 is ~4 mm at 2-3 m: pixels whose
-// nearest vertex is farther, in the first iterations of a frame, at silhouettes and where vertices are
-// sparse) go to a queue that the tail kernels drain with a group of lanes per pixel (a warp for one session,
-// 4 lanes in a batch), the lanes splitting the next rings' buckets and combining (d^2, index) keys with a
-// group min.
+// k_associate: rings 0..kRingsPerThread by the pixel's own thread or by four lanes (see there).  Pixels still open
+// after that (the bound of ring 1 is ~4 mm at 2-3 m: pixels whose nearest vertex is farther, in the first iterations
+// of a frame, at silhouettes and where vertices are sparse) go to a queue that the tail kernels drain with a group of
+// lanes per pixel (a warp for one session, kBatchTailLanes lanes in a batch), the lanes splitting the next rings'
+// buckets and combining (d^2, index) keys with a group min.
 // The pixel's offset p - v_i is added to the vertex's fixed-point sums (integer atomics: the sums do
 // not depend on the order of the additions).
 // ---------------------------------------------------------------------------------------------
@@ -730,7 +729,9 @@ void launch_associate(const Dev& d, cudaStream_t st) {
   const int nunits = ((d.cam.W + 15) / 16) * ((d.cam.H + 1) / 2);
   k_associate<<<min((nunits + kBlock / 32 - 1) / (kBlock / 32), kAssocBlocksPerSM * 152), kBlock, 0, st>>>(nullptr, nullptr,
                                                                                                    nullptr, d);
-  k_associate_tail<<<2 * 152, 32 * kTailWarps, 0, st>>>(d);
+  // (four blocks per SM: an iteration that moved the pose queues more pixels than two per SM have warps for; 200k
+  // vertices at 1280x720: 27.3 us on two, 24.1 on four, the longest launch of a frame 109 and 85)
+  k_associate_tail<<<4 * 152, 32 * kTailWarps, 0, st>>>(d);
 }
 
 // Appends this block's tile's association units to list: its pixels with a valid depth, in row-major

@@ -6,7 +6,8 @@
 //                v[V] float4, n[V] float4 (w = valid), rec[V] float4 (x,y,z, next-in-bucket bits),
 //                acc[V] Acc4 (sum of p_k - v_i in 2^-30 m, count), vispix[V] int, nbr[V] int4, rg[V] float4
 //   per face   : tris[F] int4 (a,b,c,pad), fn[F] float4 face normals
-//   per pixel  : depth[W*H] float, zbuf[W*H] u64, head[W*H] int, corr[W*H] int
+//   per pixel  : depth[W*H] float, zbuf[W*H] u64, head[W*H] int, corr[W*H] int, ppos[W*H] float4 (back-projected
+//                points, once per frame), occ (one bit per pixel: its bucket holds a vertex)
 //   solver     : partials[nblk][NP*NP] float, A[NP*NP] double, per-candidate theta / DQ tables
 #pragma once
 #include <cstdint>
