@@ -152,3 +152,33 @@ def test_result_offsets_are_the_sessions(side):
         assert np.array_equal(out["theta"], s.read("THETA"))
         assert np.array_equal(out["energy"], s.read("ENERGY"))
         assert np.abs(out["offsets"]).max() > 0
+
+
+def test_batches_around_the_in_block_queue_prefix():
+    """Up to 256 sessions a batch's tail forms the queues' prefix in its blocks, beyond that a kernel of its own does: 256
+    and 257 tiny sessions, whose pixels lie far from their few vertices so that most are queued, equal each alone."""
+    V, T = H.grid_patch(5, 4, -0.3, 0.3, -0.2, 0.2, 2.0)
+    m = H.make_model([-1], [1], [[0, 0, 1]], [[0, 0, 0]], V, T, [[0, 0, 0, 0]] * len(V), [[1, 0, 0, 0]] * len(V),
+                     W=24, H=18, fx=24.0, fy=24.0, window_half=6, cutoff=0.3, pose_iters=2, shape_iters=1)
+    n = 257
+    depth = [torch.full((18, 24), 1.95 + 0.0004 * k, dtype=torch.float32, device="cuda") for k in range(n)]
+    sess = [trk.Session(m) for _ in range(n)]
+    alone = []
+    for s, d in zip(sess, depth):
+        s.set_pose(np.zeros(1))
+        out = s.track_frame(d.cpu().numpy())
+        alone.append((out["theta"], out["offsets"], out["energy"], s.read("CORR")))
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for count in (256, 257):
+        for s in sess:
+            s.set_pose(np.zeros(1))
+        with trk.Batch(sess[:count]) as b:
+            b.track_device([d.data_ptr() for d in depth[:count]], st.cuda_stream)
+            for k in range(count):
+                got = sess[k].read_result()
+                for x, y in zip((got["theta"], got["offsets"], got["energy"], sess[k].read("CORR")), alone[k]):
+                    assert np.array_equal(x, y), (count, k)
+    assert (alone[0][3] >= 0).sum() > 50
+    for s in sess:
+        s.close()
