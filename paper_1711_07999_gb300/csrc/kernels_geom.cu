@@ -342,18 +342,21 @@ __device__ __forceinline__ void commit_pixel(const Dev& d, int best, float3 p, f
   atomicAdd(a + 3, 1ull);
 }
 
-__device__ __forceinline__ float3 back_project(const Cam& c, int px, int py, float dep) {
-  // in FP64, then moved into the session-local frame (exact up to one FP32 rounding)
-  return make_float3((float)(((double)px - (double)c.cx) * (double)dep * c.inv_fx - (double)c.ox),
-                     (float)(((double)py - (double)c.cy) * (double)dep * c.inv_fy - (double)c.oy),
-                     (float)((double)dep - (double)c.oz));
+// The pixel's point, back-projected in FP64 and then moved into the session-local frame (exact up to one FP32 rounding),
+// x and y once per frame for its twelve or so iterations: on this GPU the ~20 FP64 operations and conversions of a
+// back-projection occupy the FP64 pipe for ~1,250 cycles per warp.
+__device__ __forceinline__ void store_point(const Dev& d, int px, int py, int k, float z) {
+  const Cam& c = d.cam;
+  d.pxy[k] = make_float2((float)(((double)px - (double)c.cx) * (double)z * c.inv_fx - (double)c.ox),
+                         (float)(((double)py - (double)c.cy) * (double)z * c.inv_fy - (double)c.oy));
 }
 
-// The pixel's point, once per frame for its twelve or so iterations: on this GPU the ~20 FP64 operations and
-// conversions of a back-projection occupy the FP64 pipe for ~1,250 cycles per warp.
-__device__ __forceinline__ void store_point(const Dev& d, int px, int py, int k, float z) {
-  const float3 p = back_project(d.cam, px, py, z);
-  d.ppos[k] = make_float4(p.x, p.y, p.z, z);
+// z is left to be formed here, which keeps 8 bytes a pixel instead of 16 (the depth is there anyway): an FP32
+// difference of two FP32 numbers is the FP64 difference rounded to FP32 (2 x 24 + 2 <= 53 bits), bit for bit.
+__device__ __forceinline__ float3 load_point(const Dev& d, int k, float& dep) {
+  const float2 xy = d.pxy[k];
+  dep = d.depth[k];
+  return make_float3(xy.x, xy.y, dep - d.cam.oz);
 }
 
 // One lane's pixel (px, py) of a warp's unit (active false: the lane has none; it still takes part in
@@ -368,9 +371,8 @@ __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, boo
   float3 p = make_float3(0.f, 0.f, 0.f);
   bool open = false;
   if (inimg) {  // (the units list pixels with a valid depth)
-    const float4 pp = d.ppos[k];
-    p = f3(pp);
-    const float dep = pp.w;
+    float dep;
+    p = load_point(d, k, dep);
     if (d.association == 1) {
       // the nearest corner of the triangle the z-buffer holds at this pixel (O(1), no queue)
       const unsigned long long key = d.zbuf[k];
@@ -425,8 +427,8 @@ __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, boo
   unsigned base = 0;
   if (lane == 0 && om) base = atomicAdd(&d.qctl[0], __popc(om));
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int2(k, best.i);
-  if (inimg && !open) d.corr[k] = best.i;
+  if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = k;
+  if (inimg) d.corr[k] = best.i;  // (of an open pixel: the nearest so far, which the tail starts from)
   const bool done = !open && best.i >= 0;
   if (done) commit_pixel(d, best.i, p, best.v);
   const unsigned m = __ballot_sync(0xffffffffu, done);
@@ -448,9 +450,7 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
   float3 p = make_float3(0.f, 0.f, 0.f);
   float dep = 0.f;
   if (inimg) {
-    const float4 pp = d.ppos[k];
-    p = f3(pp);
-    dep = pp.w;
+    p = load_point(d, k, dep);
     const int q[3] = {ring_bucket(px, py, 1, 2 * sub, c.W, c.H), ring_bucket(px, py, 1, 2 * sub + 1, c.W, c.H),
                       sub == 3 ? k : -1};
     scan_group<3, false>(d, q, p, tau2, best);
@@ -473,8 +473,8 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
   if (lane == 0 && om) base = atomicAdd(&d.qctl[0], __popc(om));
   base = __shfl_sync(0xffffffffu, base, 0);
   if (sub == 0) {
-    if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int2(k, nearest);
-    else if (inimg) d.corr[k] = nearest;
+    if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = k;
+    if (inimg) d.corr[k] = nearest;
   }
   const bool done = inimg && !open && nearest >= 0 && mine == key;  // the lane that holds the nearest
   if (done) commit_pixel(d, best.i, p, best.v);
@@ -503,13 +503,12 @@ template <int GL, int PL, bool kRows>
 __device__ __forceinline__ bool tail_item(const Dev& d, unsigned item, int gl, unsigned gmask) {
   const Cam& c = d.cam;
   const float tau2 = c.tau * c.tau;
-  const int2 e = d.queue[item];
-  const int k = e.x, W = c.W, H = c.H, px = k % W, py = k / W;
-  const float4 pp = d.ppos[k];
-  const float dep = pp.w;
-  const float3 p = f3(pp);
+  const int k = d.queue[item], W = c.W, H = c.H, px = k % W, py = k / W;
+  const int near = d.corr[k];
+  float dep;
+  const float3 p = load_point(d, k, dep);
   Best w{-1, 0.f, make_float3(0.f, 0.f, 0.f)};
-  if (e.y >= 0) consider(e.y, p, d.v[e.y], tau2, w);  // the nearest so far (its record's bits)
+  if (near >= 0) consider(near, p, d.v[near], tau2, w);  // the nearest so far (its record's bits)
   unsigned long long key = key_of(w.i, w.d2);
   // several rings at a time: scanning rings past the one whose bound ends the search only confirms the
   // argmin, so the result is the same

@@ -1745,7 +1745,7 @@ __device__ __forceinline__ void cg_init_impl(const Dev& d, BlockPos bp, int src,
     d.cg_x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     d.cg_r[i] = make_float4(rr.x, rr.y, rr.z, 0.f);
     d.cg_z[i] = make_float4(z.x, z.y, z.z, 0.f);
-    d.cg_p[0][i] = make_float4(z.x, z.y, z.z, 0.f);
+    d.cg_p[i] = make_float4(z.x, z.y, z.z, 0.f);
   }
   const double rz = dot3_fp64(rr, z);
   const unsigned m = __ballot_sync(0xffffffffu, inA_count != 0);
@@ -1758,23 +1758,27 @@ __device__ __forceinline__ void cg_init_impl(const Dev& d, BlockPos bp, int src,
   block_energy_to_slot(d, bp, e, slot, 1);
 }
 
+// The direction of iteration k: of odd ones in the Phi buffer that receives the result (nothing reads that before the
+// last iteration, and there each thread only its own entry, before it writes the result over it).
+__device__ __forceinline__ float4* cg_direction(const Dev& d, int src, int k) { return k & 1 ? d.phi[1 - src] : d.cg_p; }
+
 // Iteration k > 0: p = z + beta p first (the neighbours' too, each formed from its z and old p, so that the
 // direction needs no pass of its own; p is written to the other buffer).  Ap = (B - lambda_N Adj) p;
 // alpha = r.z / p.Ap (0 and stop on a breakdown).
-__device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp, int k) {
+__device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp, int src, int k) {
   const int i = bp.x * kBlock + threadIdx.x;
   float3 p = make_float3(0.f, 0.f, 0.f), ap = p;
   if (i < d.V) {
     const float beta = (float)d.cg[2];
-    const float4* old = d.cg_p[(k - 1) & 1];
+    const float4* old = cg_direction(d, src, k - 1);
     auto direction = [&](int j) {
-      if (k == 0) return f3(d.cg_p[0][j]);
+      if (k == 0) return f3(d.cg_p[j]);
       const float3 z = f3(d.cg_z[j]), q = f3(old[j]);
       return make_float3(z.x + beta * q.x, z.y + beta * q.y, z.z + beta * q.z);
     };
     const float4 rg = d.rg[i];
     p = direction(i);
-    if (k > 0) d.cg_p[k & 1][i] = make_float4(p.x, p.y, p.z, 0.f);
+    if (k > 0) cg_direction(d, src, k)[i] = make_float4(p.x, p.y, p.z, 0.f);
     const int a0 = d.adj_off[i], a1 = d.adj_off[i + 1];
     ap = block_apply(f3(rg), d.lambda_phi + d.lambda_N * (float)(a1 - a0), d.lambda_w, p);
     for_neighbours(d, a0, a1, direction, [&](float3 q) {
@@ -1791,15 +1795,15 @@ __device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp, int k) 
   }
 }
 
-// x += alpha p, r -= alpha Ap, z = B^-1 r; beta = r.z_new / r.z.  The last iteration (out >= 0): phi[out] =
-// phi[1 - out] + x.
-__device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int k, int out) {
+// x += alpha p, r -= alpha Ap, z = B^-1 r; beta = r.z_new / r.z.  The last iteration: phi[1 - src] =
+// phi[src] + x.
+__device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int src, int k, bool last) {
   const int i = bp.x * kBlock + threadIdx.x;
   float3 r = make_float3(0.f, 0.f, 0.f), z = r;
   if (i < d.V) {
     const float alpha = (float)d.cg[1];
     const float4 rg = d.rg[i];
-    const float3 p = f3(d.cg_p[k & 1][i]), ap = f3(d.cg_ap[i]);
+    const float3 p = f3(cg_direction(d, src, k)[i]), ap = f3(d.cg_ap[i]);
     float3 x = f3(d.cg_x[i]);
     r = f3(d.cg_r[i]);
     x.x += alpha * p.x; x.y += alpha * p.y; x.z += alpha * p.z;
@@ -1809,9 +1813,9 @@ __device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int k,
     d.cg_x[i] = make_float4(x.x, x.y, x.z, 0.f);
     d.cg_r[i] = make_float4(r.x, r.y, r.z, 0.f);
     d.cg_z[i] = make_float4(z.x, z.y, z.z, 0.f);
-    if (out >= 0) {
-      const float4 f = d.phi[1 - out][i];
-      d.phi[out][i] = make_float4(f.x + x.x, f.y + x.y, f.z + x.z, 0.f);
+    if (last) {
+      const float4 f = d.phi[src][i];
+      d.phi[1 - src][i] = make_float4(f.x + x.x, f.y + x.y, f.z + x.z, 0.f);
     }
   }
   const double rz = dot3_fp64(r, z);
@@ -1835,10 +1839,10 @@ __device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int k,
   }
 #define ARGS_k_cg_init , int src, int slot
 #define CALL_k_cg_init , src, slot
-#define ARGS_k_cg_apply , int k
-#define CALL_k_cg_apply , k
-#define ARGS_k_cg_update , int k, int out
-#define CALL_k_cg_update , k, out
+#define ARGS_k_cg_apply , int src, int k
+#define CALL_k_cg_apply , src, k
+#define ARGS_k_cg_update , int src, int k, bool last
+#define CALL_k_cg_update , src, k, last
 TRK_CG_KERNEL(k_cg_init, cg_init_impl)
 TRK_CG_KERNEL(k_cg_apply, cg_apply_impl)
 TRK_CG_KERNEL(k_cg_update, cg_update_impl)
@@ -1849,8 +1853,8 @@ static void launch_shape_pcg(const BatchGrid& g, int n, const Dev& d0, int max_l
   if (n <= 0) return;
   k_cg_init<<<n, kBlock, max_links * sizeof(DQ), st>>>(g, d0, src, slot);
   for (int k = 0; k < iters; ++k) {
-    k_cg_apply<<<n, kBlock, 0, st>>>(g, d0, k);
-    k_cg_update<<<n, kBlock, 0, st>>>(g, d0, k, k + 1 < iters ? -1 : 1 - src);
+    k_cg_apply<<<n, kBlock, 0, st>>>(g, d0, src, k);
+    k_cg_update<<<n, kBlock, 0, st>>>(g, d0, src, k, k + 1 == iters);
   }
 }
 

@@ -529,15 +529,15 @@ void carve_all(trk_session* s) {
   carve(s, &d.lm_ok, 2 * kCandidates);
   carve(s, &d.v, V); carve(s, &d.n, V); carve(s, &d.fn, F); carve(s, &d.rec, V);
   carve(s, &d.head, npx); carve(s, &d.zbuf, npx); carve(s, &d.corr, npx);
-  carve(s, &d.pixrec, npx); carve(s, &d.queue, npx); carve(s, &d.qctl, 4); carve(s, &d.ppos, npx);
+  carve(s, &d.pixrec, npx); carve(s, &d.queue, npx); carve(s, &d.qctl, 4); carve(s, &d.pxy, npx);
   carve(s, &d.occ, (size_t)d.cam.H * occ_row(d.cam.W));
   carve(s, &d.units, (size_t)kUnitsPerTile * ((d.cam.W + 15) / 16) * ((d.cam.H + 15) / 16));
   carve(s, &d.acc, V); carve(s, &d.vispix, V); carve(s, &d.rg, V); carve(s, &d.phi0, V);
   carve(s, &dadj_off, V + 1); carve(s, &dadj, s->hm.adj.size());
-  d.cg_x = d.cg_r = d.cg_z = d.cg_p[0] = d.cg_p[1] = d.cg_ap = nullptr;
+  d.cg_x = d.cg_r = d.cg_z = d.cg_p = d.cg_ap = nullptr;
   if (prm.shape_solver == 1) {
     carve(s, &d.cg_x, V); carve(s, &d.cg_r, V); carve(s, &d.cg_z, V);
-    carve(s, &d.cg_p[0], V); carve(s, &d.cg_p[1], V); carve(s, &d.cg_ap, V);
+    carve(s, &d.cg_p, V); carve(s, &d.cg_ap, V);
   }
   carve(s, &d.cg, 4);
   carve(s, &ddepth, npx);

@@ -6,8 +6,8 @@
 //                v[V] float4, n[V] float4 (w = valid), rec[V] float4 (x,y,z, next-in-bucket bits),
 //                acc[V] Acc4 (sum of p_k - v_i in 2^-30 m, count), vispix[V] int, nbr[V] int4, rg[V] float4
 //   per face   : tris[F] int4 (a,b,c,pad), fn[F] float4 face normals
-//   per pixel  : depth[W*H] float, zbuf[W*H] u64, head[W*H] int, corr[W*H] int, ppos[W*H] float4 (back-projected
-//                points, once per frame), occ (one bit per pixel: its bucket holds a vertex)
+//   per pixel  : depth[W*H] float, zbuf[W*H] u64, head[W*H] int, corr[W*H] int, pxy[W*H] float2 (back-projected
+//                points, once per frame), queue[W*H] int, occ (one bit per pixel: its bucket holds a vertex)
 //   solver     : partials[nblk][NP*NP] float, A[NP*NP] double, per-candidate theta / DQ tables
 #pragma once
 #include <cstdint>
@@ -361,8 +361,8 @@ struct Dev {
   float4* pixrec;  // [W*H] first vertex inserted into each pixel's bucket: x, y, z, index bits
   int* head;
   unsigned* occ;   // [H][occ_row(W)] one bit per pixel: its bucket holds a vertex
-  float4* ppos;    // [W*H] pixels with a valid depth: back-projected point (session-local frame), depth in w
-  int2* queue;     // [W*H] pixels whose association search goes on past the thread-owned rings: (pixel, nearest so far)
+  float2* pxy;     // [W*H] pixels with a valid depth: x, y of the back-projected point (session-local frame)
+  int* queue;      // [W*H] pixels whose association search goes on past the thread-owned rings (nearest so far: corr)
   unsigned int* qctl;  // [0] queued pixels, [1] next queue entry to take, [2] association units, [3] unused
   AssocUnit* units;  // [8 ceil(W/16) ceil(H/16)] association units of the frame (up to 32 valid pixels of a tile)
   unsigned long long* zbuf;
@@ -389,7 +389,7 @@ struct Dev {
   int association;        // 0 window search, 1 nearest corner of the rasterised triangle
   const int* adj_off;     // [V + 1] neighbourhood edges of each vertex in both directions (CSR) ...
   const int* adj;         // ... sorted by vertex index
-  float4 *cg_x, *cg_r, *cg_z, *cg_p[2], *cg_ap;  // [V] PCG vectors (the direction of iteration k in cg_p[k & 1])
+  float4 *cg_x, *cg_r, *cg_z, *cg_p, *cg_ap;  // [V] PCG vectors (the direction of odd iterations: in the other phi)
   double* cg;             // [4] rz, alpha, beta, stopped
 };
 
