@@ -15,8 +15,7 @@
 namespace trk {
 
 constexpr int kJBlock = 256;      // rows that make a CTA worth having (the grid's rule)
-constexpr int kJStage = 16;       // rows per pipeline stage
-constexpr int kJStages = 4;
+constexpr int kJStages = 4;       // pipeline stages
 constexpr int kJLoaders = 128;    // threads that only load
 constexpr int kJMaxBlocks = 296;
 
@@ -26,13 +25,18 @@ constexpr int kJMaxBlocks = 296;
 // the tiles.  Per SM and row that is bound by the FMAs' operand reads (fma.rn.f32x2: about 3 cycles per
 // warp and sub-partition, measured) and by shared memory returning 32 floats per cycle: 8 x 4 tiles take
 // 96 and 96 cycles at 73 columns (8 x 8 tiles: 113, and only half of the sub-partitions get one of the
-// CTA's two warps of them, 206 in all; 4 x 4 ones: 84 and 112).  Up to 32 columns, where the rows of a CTA
-// are a chain that nothing else overlaps, 4 x 4 tiles have the shortest one (25 cycles a row).  The row
-// loop is unrolled over a whole stage so that its loads run ahead (62 cycles a row unrolled by 4).  Two
-// further warps copy the rows ahead with cp.async (16-byte pieces where base and ld allow, else 4-byte
-// ones) through four stages, one barrier per 16 rows; missing rows of the last stage are zeros.  One million
-// rows of 73 columns: 806 -> 198 us.  The version before formed the whole square from 5 x 5 tiles (scalar
-// reads) and loaded between its two barriers per 64 rows.
+// CTA's two warps of them, 206 in all; 4 x 4 ones: 84 and 112).  Fewer columns leave a CTA one to three warps
+// whose rows are a chain that nothing else overlaps; there 4 x 4 tiles have the shorter one.  The row loop is
+// unrolled by 16 so that its loads run ahead (62 cycles a row unrolled by 4).
+//
+// Four further warps copy the rows ahead with cp.async (16-byte pieces where base and ld allow, else 4-byte
+// ones) through four stages, one barrier per STAGE rows; missing rows of the last stage are zeros.  Rows lie
+// W floats apart, so that narrow ones share the memory among more of them: with 16 rows a stage whatever
+// their width, up to 16 columns a stage was little but its barrier and a quarter of the loaders' lanes
+// had a piece.  A row's pieces are spread over kLanes lanes.
+// A call on one million rows, microseconds (64 rows staged between two barriers and the whole square formed; 16 rows
+// a stage at any width; this): 8 columns 105, 115, 64; 32: 165, 112, 90; 48: 477, 155, 120; 73: 838, 221,
+// 217.  20,000 rows of 8 columns: 15.6, 17.6, 15.5.
 template <int TA, int TB>
 struct JTiles {
   static __host__ __device__ int cols(int nc) { return (nc + TB - 1) / TB; }
@@ -65,14 +69,17 @@ __device__ __forceinline__ void load_floats(const float* p, float (&v)[N]) {
   }
 }
 
-template <int TA, int TB>
+template <int TA, int TB, int W, int STAGE>
 __global__ void __launch_bounds__(kJLoaders + 128) k_jtj_rows(const float* __restrict__ rows, int n, int nc, int ld,
                                                             int rows_per_block, bool vec, float* __restrict__ partial) {
-  constexpr int W = kMaxNP;  // row stride: 16-byte rows; tiles past nc read the row's leftovers, which count nowhere
-  __shared__ __align__(16) float st[kJStages][kJStage][W];
+  // (W >= nc, a multiple of 16; tiles past nc read a row's leftovers, which count nowhere)
+  constexpr int kLanes = W <= 16 ? 4 : W <= 32 ? 8 : W <= 64 ? 16 : 32;
+  constexpr int kRowsAtOnce = kJLoaders / kLanes, kRowsEach = STAGE / kRowsAtOnce;
+  static_assert(STAGE % kRowsAtOnce == 0 && STAGE % 16 == 0, "whole rounds of the loaders and of the row loop");
+  __shared__ __align__(16) float st[kJStages][STAGE][W];
   const int tid = threadIdx.x, nthr = blockDim.x, ncomp = nthr - kJLoaders;
   const int r0 = blockIdx.x * rows_per_block, r1 = min(n, r0 + rows_per_block);
-  const int nst = r1 > r0 ? (r1 - r0 + kJStage - 1) / kJStage : 0;
+  const int nst = r1 > r0 ? (r1 - r0 + STAGE - 1) / STAGE : 0;
   // this thread's tile
   int ti = 0, tj = tid;
   const int ncols = JTiles<TA, TB>::cols(nc);
@@ -82,30 +89,28 @@ __global__ void __launch_bounds__(kJLoaders + 128) k_jtj_rows(const float* __res
   }
   tj += TA * ti / TB;
   const bool comp = tid < ncomp && TA * ti < nc;
-  const int pieces = vec ? (nc + 3) / 4 : nc, lw = (tid - ncomp) >> 5;
+  const int pieces = vec ? (nc + 3) / 4 : nc, lt = tid - ncomp;
   auto load = [&](int q) {  // stage q, by the loader threads
-    const int base = r0 + q * kJStage, cnt = min(kJStage, r1 - base);
-    // a lane per piece, a warp per row; few instructions (a stage is one warp's chain of them)
-    constexpr int kWarps = kJLoaders / 32, kRowsEach = kJStage / kWarps;
-    for (int piece = tid & 31; piece < pieces; piece += 32) {
+    const int base = r0 + q * STAGE, cnt = min(STAGE, r1 - base), row = lt / kLanes;
+    for (int piece = lt % kLanes; piece < pieces; piece += kLanes) {
       const int col = vec ? 4 * piece : piece, bytes = vec ? 4 * min(4, nc - col) : 4;
-      const float* src = rows + (size_t)(base + lw) * ld + col;
-      float* dst = &st[q % kJStages][lw][col];
-      const size_t step = (size_t)kWarps * ld;
-      if (cnt == kJStage) {
+      const float* src = rows + (size_t)(base + row) * ld + col;
+      float* dst = &st[q % kJStages][row][col];
+      const size_t step = (size_t)kRowsAtOnce * ld;
+      if (cnt == STAGE) {
 #pragma unroll
         for (int i = 0; i < kRowsEach; ++i) {
-          if (vec) cp_async16_part(dst + i * kWarps * W, src + i * step, bytes);
-          else cp_async4(dst + i * kWarps * W, src + i * step);
+          if (vec) cp_async16_part(dst + i * kRowsAtOnce * W, src + i * step, bytes);
+          else cp_async4(dst + i * kRowsAtOnce * W, src + i * step);
         }
       } else {
-        for (int i = 0; lw + i * kWarps < cnt; ++i) {
-          if (vec) cp_async16_part(dst + i * kWarps * W, src + i * step, bytes);
-          else cp_async4(dst + i * kWarps * W, src + i * step);
+        for (int i = 0; row + i * kRowsAtOnce < cnt; ++i) {
+          if (vec) cp_async16_part(dst + i * kRowsAtOnce * W, src + i * step, bytes);
+          else cp_async4(dst + i * kRowsAtOnce * W, src + i * step);
         }
       }
     }
-    for (int e = cnt * W + tid - ncomp; e < kJStage * W; e += kJLoaders) st[q % kJStages][0][e] = 0.f;
+    for (int e = cnt * W + lt; e < STAGE * W; e += kJLoaders) st[q % kJStages][0][e] = 0.f;
   };
   unsigned long long acc[TA][TB / 2];
 #pragma unroll
@@ -127,8 +132,8 @@ __global__ void __launch_bounds__(kJLoaders + 128) k_jtj_rows(const float* __res
     } else if (comp) {
       const float* pa = &st[q % kJStages][0][TA * ti];
       const float* pb = &st[q % kJStages][0][TB * tj];
-#pragma unroll
-      for (int s = 0; s < kJStage; ++s) {
+#pragma unroll 16
+      for (int s = 0; s < STAGE; ++s) {
         float ra[TA], rb[TB];
         load_floats(pa + s * W, ra);
         load_floats(pb + s * W, rb);
@@ -222,10 +227,10 @@ static void launch_reduce(const float* partial, int nblk, int nc, double* out, c
   k_jtj_reduce<kUpper><<<(total + 31) / 32, 32 * std::min(32, std::max(1, (nblk + 1) / 2)), 0, st>>>(partial, nblk, nc, out);
 }
 
-template <int TA, int TB>
+template <int TA, int TB, int W, int STAGE>
 static void launch_rows(const float* rows, int n, int nc, int ld, int nblk, int rpb, bool vec, float* partial,
                         cudaStream_t st) {
-  k_jtj_rows<TA, TB><<<nblk, JTiles<TA, TB>::compute_threads(nc) + kJLoaders, 0, st>>>(rows, n, nc, ld, rpb, vec, partial);
+  k_jtj_rows<TA, TB, W, STAGE><<<nblk, JTiles<TA, TB>::compute_threads(nc) + kJLoaders, 0, st>>>(rows, n, nc, ld, rpb, vec, partial);
 }
 
 // Launches the two kernels with nblk CTAs and the given partial buffer (nblk * nc * nc floats).
@@ -233,8 +238,12 @@ cudaError_t jtj_rows_launch(const float* rows, int n, int nc, int ld, double* ou
                             cudaStream_t st) {
   const int rpb = (n + nblk - 1) / nblk;
   const bool vec = ld % 4 == 0 && reinterpret_cast<uintptr_t>(rows) % 16 == 0;
-  if (nc > 32) launch_rows<8, 4>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
-  else launch_rows<4, 4>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
+  // 4 x 4 tiles up to 48 columns: there 3,001, 50,010 and a million rows take 13, 18.6 and 120 us, with 8 x 4 ones
+  // 16.6, 22.7 and 155; at 56 columns 15, 22.7 and 159 against 16.6, 22.8 and 156
+  if (nc <= 16) launch_rows<4, 4, 16, 64>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
+  else if (nc <= 32) launch_rows<4, 4, 32, 32>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
+  else if (nc <= 48) launch_rows<4, 4, 48, 32>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
+  else launch_rows<8, 4, kMaxNP, 16>(rows, n, nc, ld, nblk, rpb, vec, partial, st);
   launch_reduce<true>(partial, nblk, nc, out, st);
   return cudaGetLastError();
 }
