@@ -1673,23 +1673,6 @@ __device__ __forceinline__ double dot3_fp64(float3 a, float3 b) {
   return ax * bx + ay * by + az * bz;
 }
 
-// Sums f(neighbour) over the neighbourhood edges [a0, a1) of a vertex in order, eight loads in flight.
-template <typename Load, typename Add>
-__device__ __forceinline__ void for_neighbours(const Dev& d, int a0, int a1, Load load, Add add) {
-  for (int t = a0; t < a1; t += 8) {
-    int j[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) j[u] = t + u < a1 ? d.adj[t + u] : -1;
-    float3 q[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (j[u] >= 0) q[u] = load(j[u]);
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (j[u] >= 0) add(q[u]);
-  }
-}
-
 // B_i = M_i + lambda_w diag(M_i), M_i = g g^T + c I (g = 0 outside A): B_i p and B_i^-1 p.
 __device__ __forceinline__ float3 block_apply(float3 g, float c, float lw, float3 p) {
   const float gp = g.x * p.x + g.y * p.y + g.z * p.z;
@@ -1734,8 +1717,10 @@ __device__ __forceinline__ void cg_init_impl(const Dev& d, BlockPos bp, int src,
     }
     float3 sd = make_float3(0.f, 0.f, 0.f);
     const int a0 = d.adj_off[i], a1 = d.adj_off[i + 1];
-    for_neighbours(d, a0, a1, [&](int j) { return f3(phi[j]); },
-                   [&](float3 q) { sd.x += pi.x - q.x; sd.y += pi.y - q.y; sd.z += pi.z - q.z; });
+    for (int t = a0; t < a1; ++t) {
+      const float3 q = f3(phi[d.adj[t]]);
+      sd.x += pi.x - q.x; sd.y += pi.y - q.y; sd.z += pi.z - q.z;
+    }
     rr = make_float3(-(g.x * r + d.lambda_phi * pi.x + d.lambda_N * sd.x),
                      -(g.y * r + d.lambda_phi * pi.y + d.lambda_N * sd.y),
                      -(g.z * r + d.lambda_phi * pi.z + d.lambda_N * sd.z));
@@ -1764,7 +1749,10 @@ __device__ __forceinline__ float4* cg_direction(const Dev& d, int src, int k) { 
 
 // Iteration k > 0: p = z + beta p first (the neighbours' too, each formed from its z and old p, so that the
 // direction needs no pass of its own; p is written to the other buffer).  Ap = (B - lambda_N Adj) p;
-// alpha = r.z / p.Ap (0 and stop on a breakdown).
+// alpha = r.z / p.Ap (0 and stop on a breakdown).  Bound by the latency of its gathers, which warps hide
+// better than loads ahead do: one neighbour at a time in 32 registers, eight blocks per SM (a coupled step of
+// eight iterations at 55k and 200k vertices and of sixteen sessions of 50k: 180, 307 and 769 us; eight
+// neighbours ahead in 80 registers: 188, 322 and 904; a pass of its own for p, in 40: 213, 330 and 796).
 __device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp, int src, int k) {
   const int i = bp.x * kBlock + threadIdx.x;
   float3 p = make_float3(0.f, 0.f, 0.f), ap = p;
@@ -1781,9 +1769,11 @@ __device__ __forceinline__ void cg_apply_impl(const Dev& d, BlockPos bp, int src
     if (k > 0) cg_direction(d, src, k)[i] = make_float4(p.x, p.y, p.z, 0.f);
     const int a0 = d.adj_off[i], a1 = d.adj_off[i + 1];
     ap = block_apply(f3(rg), d.lambda_phi + d.lambda_N * (float)(a1 - a0), d.lambda_w, p);
-    for_neighbours(d, a0, a1, direction, [&](float3 q) {
+#pragma unroll 1
+    for (int t = a0; t < a1; ++t) {
+      const float3 q = direction(d.adj[t]);
       ap.x -= d.lambda_N * q.x; ap.y -= d.lambda_N * q.y; ap.z -= d.lambda_N * q.z;
-    });
+    }
     d.cg_ap[i] = make_float4(ap.x, ap.y, ap.z, 0.f);
   }
   const double pap = dot3_fp64(p, ap);
@@ -1828,8 +1818,8 @@ __device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int sr
   }
 }
 
-#define TRK_CG_KERNEL(name, impl, ...)                                                     \
-  __global__ void __launch_bounds__(kBlock) name(BatchGrid g, Dev d0 ARGS_##name) {         \
+#define TRK_CG_KERNEL(name, impl, blocks_per_sm)                                           \
+  __global__ void __launch_bounds__(kBlock, blocks_per_sm) name(BatchGrid g, Dev d0 ARGS_##name) {         \
     if (g.map == nullptr) {                                                                  \
       impl(d0, grid_pos() CALL_##name);                                                      \
       return;                                                                                \
@@ -1843,9 +1833,9 @@ __device__ __forceinline__ void cg_update_impl(const Dev& d, BlockPos bp, int sr
 #define CALL_k_cg_apply , src, k
 #define ARGS_k_cg_update , int src, int k, bool last
 #define CALL_k_cg_update , src, k, last
-TRK_CG_KERNEL(k_cg_init, cg_init_impl)
-TRK_CG_KERNEL(k_cg_apply, cg_apply_impl)
-TRK_CG_KERNEL(k_cg_update, cg_update_impl)
+TRK_CG_KERNEL(k_cg_init, cg_init_impl, 5)
+TRK_CG_KERNEL(k_cg_apply, cg_apply_impl, 8)
+TRK_CG_KERNEL(k_cg_update, cg_update_impl, 8)
 
 // The whole coupled step (g, n: the block table and its size for a batch; kSingle and nblk_v alone).
 static void launch_shape_pcg(const BatchGrid& g, int n, const Dev& d0, int max_links, int iters, int src, int slot,
