@@ -770,7 +770,8 @@ void launch_normal_equations(const Dev& d, int phi_buf, int slot, cudaStream_t s
 // substitutions 2 x 4.7k, two FP64 residuals 2 x 2.9k (the FP64 pipe's rate), FK 9k.  Measured per launch,
 // humanoid 50k: 34.9 -> 20 us (a frame of ten iterations 1,406 -> 1,259 us).
 // ---------------------------------------------------------------------------------------------
-constexpr int kSolveThreads = 256;
+constexpr int kSolveThreads = 256, kSolveBlocksPerSM = 2;
+constexpr int kCrowdThreads = 192, kCrowdBlocksPerSM = 3;  // of a batch that takes fewer waves so
 constexpr int kMaxRefine = 8;
 
 __device__ void chol_solve_fp64(double* M, int ld, double* b, int P, int& fail_out) {
@@ -869,7 +870,7 @@ __device__ bool chol_blocked(float* F, float* G, float* ivd, int Pp) {
   // this thread's tiles (2 rows x 4 columns) of the trailing triangle, relative to its corner: row pairs in
   // order, pair i with i / 2 + 1 tiles, so the rows 4 m .. 4 m + 3 hold 2 (m + 1) from tile m (m + 1) on
   // (at most 18 x 19 tiles for 72 rows)
-  static_assert(2 * kSolveThreads >= 18 * 19, "two tiles per thread cover the largest trailing triangle");
+  static_assert(2 * kCrowdThreads >= 18 * 19, "two tiles per thread cover the largest trailing triangle");
   int tile[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -1002,15 +1003,15 @@ __device__ __forceinline__ void solve_block(const float* G, const float* const (
 }
 
 // y <- (L L^T)^-1 y with the factor of chol_blocked, by one warp without block barriers: lane l holds rows
-// l + 32 k; z (16-byte aligned, kMaxPad) is scratch.
+// l + 32 k; z (16-byte aligned, kMaxPad) is scratch; G has g_rows rows.
 template <int SETS>
 __device__ __forceinline__ void solve_warp(const float* G, const float* ivd, float (&y)[SETS], float* z,
-                                           int Pp) {
+                                           int Pp, int g_rows) {
   const int lane = threadIdx.x & 31;
   float a[kBlk][kBlk], iv[kBlk], an[kBlk][kBlk], ivn[kBlk];
   const float* rows[SETS];  // this lane's rows of G
 #pragma unroll
-  for (int k = 0; k < SETS; ++k) rows[k] = G + fidx(min(32 * k + lane, kMaxPad - 1), 0);
+  for (int k = 0; k < SETS; ++k) rows[k] = G + fidx(min(32 * k + lane, g_rows - 1), 0);
   load_diag(G, 0, a);
   load8(ivd, iv);
 #pragma unroll 1
@@ -1038,12 +1039,13 @@ __device__ __forceinline__ void solve_warp(const float* G, const float* ivd, flo
 
 // ys <- (L L^T)^-1 ys by one warp.
 template <int SETS>
-__device__ __forceinline__ void solve_rows(const float* G, const float* ivd, float* ys, float* z, int P, int Pp) {
+__device__ __forceinline__ void solve_rows(const float* G, const float* ivd, float* ys, float* z, int P, int Pp,
+                                           int g_rows) {
   const int lane = threadIdx.x & 31;
   float y[SETS];
 #pragma unroll
   for (int k = 0; k < SETS; ++k) y[k] = lane + 32 * k < P ? ys[lane + 32 * k] : 0.f;
-  solve_warp<SETS>(G, ivd, y, z, Pp);
+  solve_warp<SETS>(G, ivd, y, z, Pp, g_rows);
 #pragma unroll
   for (int k = 0; k < SETS; ++k)
     if (lane + 32 * k < P) ys[lane + 32 * k] = y[k];
@@ -1062,13 +1064,28 @@ __device__ __forceinline__ float to_float_rn(double x, bool& other) {
   return __uint_as_float((zero ? 0u : t + up) | (hi & 0x80000000u));
 }
 
-// Byte offset of the link table in the solve's dynamic shared memory: behind F (P padded to the block, rows
-// of kFRow), G (kMaxPad rows: the substitution's lanes read past the padded P), M and six P-vectors.
-__host__ __device__ inline size_t lm_solve_table_offset(int P) {
-  const size_t Pp = (P + kBlk - 1) / kBlk * kBlk, NP = P + 1;
-  return (((fidx((int)Pp, 0) + fidx(kMaxPad, 0)) * sizeof(float) + (NP * NP + 6 * (size_t)P) * sizeof(double)) + 15) & ~(size_t)15;
-}
+// The solve's dynamic shared memory: F (P padded to the block, rows of kFRow), G (kMaxPad rows: the substitution's lanes
+// read past the padded P), M, six P-vectors, then the link table and the links' dual quaternions.  kLate: G without the
+// rows past the padded P, and the last two in F's place, once the factor has used it up.
+constexpr int kLinkTableBytes = (sizeof(LinkTable) + 15) & ~15;
+__host__ __device__ constexpr int padded(int P) { return (P + kBlk - 1) / kBlk * kBlk; }
+template <bool kLate>
+struct SolveLayout {
+  static __host__ __device__ constexpr int g_rows(int P) { return kLate ? padded(P) : kMaxPad; }
+  static __host__ __device__ constexpr int links(int P) { return kLinkTableBytes + P * (int)sizeof(DQ); }
+  static __host__ __device__ constexpr int g(int P) {  // byte offsets; F at 0
+    const int f = fidx(padded(P), 0) * (int)sizeof(float);
+    return kLate && links(P) > f ? links(P) : f;
+  }
+  static __host__ __device__ constexpr int m(int P) { return g(P) + fidx(g_rows(P), 0) * (int)sizeof(float); }
+  static __host__ __device__ constexpr int end(int P) {
+    return (m(P) + ((P + 1) * (P + 1) + 6 * P) * (int)sizeof(double) + 15) & ~15;
+  }
+  static __host__ __device__ constexpr int table(int P) { return kLate ? 0 : end(P); }
+  static __host__ __device__ constexpr int bytes(int P) { return kLate ? end(P) : end(P) + links(P); }
+};
 
+template <bool kLate>
 __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(16) float ivd[kMaxPad], zs[kMaxPad];
@@ -1076,17 +1093,18 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   const int P = d.L, NP = d.NP, c = bp.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int Pp = (P + kBlk - 1) / kBlk * kBlk;
   float* F = reinterpret_cast<float*>(smem_raw);  // FP32 scaled system (used up by the factor)
-  float* G = F + fidx(Pp, 0);                     // its Cholesky factor
+  using Layout = SolveLayout<kLate>;
+  float* G = reinterpret_cast<float*>(smem_raw + Layout::g(P));  // its Cholesky factor
   // [NP][NP] as the reduction left it (J^T J, J^T r in column P), then the FP64 system for the residuals
-  double* M = reinterpret_cast<double*>(G + fidx(kMaxPad, 0));
+  double* M = reinterpret_cast<double*>(smem_raw + Layout::m(P));
   double* x = M + NP * NP;
   double* res = x + P;
   double* b = res + P;
   double* dg = b + P;
   double* p2 = dg + P;  // (lambda_s S_kk)^2
   double* th = p2 + P;  // Theta
-  LinkTable* lt = reinterpret_cast<LinkTable*>(smem_raw + lm_solve_table_offset(P));
-  DQ* H0 = reinterpret_cast<DQ*>(reinterpret_cast<unsigned char*>(lt) + ((sizeof(LinkTable) + 15) & ~(size_t)15));
+  LinkTable* lt = reinterpret_cast<LinkTable*>(smem_raw + Layout::table(P));
+  DQ* H0 = reinterpret_cast<DQ*>(smem_raw + Layout::table(P) + kLinkTableBytes);
   __shared__ unsigned rmax_bits[2], bmax_bits;  // rmax: one slot per refinement parity
   __shared__ unsigned char frz[kMaxPad];
   __shared__ int any_frz;
@@ -1097,8 +1115,11 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
     cp_async8(p2 + r, d.prior2 + r);
     cp_async8(th + r, d.theta + r);
   }
-  for (int t = tid; t < (int)(sizeof(LinkTable) / 16); t += nt)
-    cp_async16(reinterpret_cast<char*>(lt) + 16 * t, reinterpret_cast<const char*>(d.links) + 16 * t);
+  auto load_links = [&] {
+    for (int t = tid; t < (int)(sizeof(LinkTable) / 16); t += nt)
+      cp_async16(reinterpret_cast<char*>(lt) + 16 * t, reinterpret_cast<const char*>(d.links) + 16 * t);
+  };
+  if (!kLate) load_links();
   double lam = *d.lam;
   for (int t = 0; t < c; ++t) lam = fmin(lam * 10.0, 1e7);
   if (tid == 0) bmax_bits = rmax_bits[0] = any_frz = 0;
@@ -1111,12 +1132,13 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   // ---- setup: M = A + diag(prior + lambda dg) (FP64), frozen rows/columns -> identity; scale D in FP32
   // (an FP64 instruction occupies its sub-partition's pipe for 64 cycles per warp: the two halves of the
   // block take a part of the vectors each)
-  static_assert(kSolveThreads / 2 >= kMaxPad, "half a block covers the rows");
+  static_assert(kCrowdThreads / 2 >= kMaxPad, "half a block covers the rows");
   {
-    const int r = tid & (kSolveThreads / 2 - 1);
+    constexpr int half = (kLate ? kCrowdThreads : kSolveThreads) / 2;
+    const int r = tid < half ? tid : tid - half;
     if (r < P) {
       double& mrr = M[(size_t)r * NP + r];
-      if (tid < kSolveThreads / 2) {
+      if (tid < half) {
         const double dgr = mrr + p2[r];
         const bool fr = dgr == 0.0;
         frz[r] = fr;
@@ -1196,16 +1218,17 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
   }
   __syncthreads();
   // ---- FP32 factor of D M D, padded with identity rows to a multiple of the block size
-  const bool ok32 = chol_blocked(F, G, ivd, Pp);
+  const bool ok32 = chol_blocked(F, G, ivd, Pp);  // (its last barrier: nothing reads F any more)
+  if (kLate) load_links();
   // ---- iterative refinement: x += D (D M D)^-1 D (b - M x), residual in FP64
   int iters = 0;
   bool converged = false;
   const float bmax = __uint_as_float(bmax_bits);
   for (int it = 0; it < kMaxRefine && ok32; ++it) {
     if (warp == 0) {
-      if (Pp <= 32) solve_rows<1>(G, ivd, ys, zs, P, Pp);
-      else if (Pp <= 64) solve_rows<2>(G, ivd, ys, zs, P, Pp);
-      else solve_rows<3>(G, ivd, ys, zs, P, Pp);
+      if (Pp <= 32) solve_rows<1>(G, ivd, ys, zs, P, Pp, Layout::g_rows(P));
+      else if (Pp <= 64) solve_rows<2>(G, ivd, ys, zs, P, Pp, Layout::g_rows(P));
+      else solve_rows<3>(G, ivd, ys, zs, P, Pp, Layout::g_rows(P));
     }
     __syncthreads();
     for (int r = tid; r < P; r += nt) x[r] += (double)sc[r] * (double)ys[r];
@@ -1257,17 +1280,20 @@ __device__ __forceinline__ void lm_solve_impl(const Dev& d, BlockPos bp) {
     d.lm_ok[c] = !fail;
     d.lm_ok[kCandidates + c] = converged ? iters : (fail ? -2 : -1);
   }
+  if (kLate) cp_async_wait_all();
   __syncthreads();
   fk_all(*lt, res, H0, d.Hd_c + (size_t)c * P, d.xi_c + (size_t)c * P * 8, 8);
 }
 
-__global__ void __launch_bounds__(kSolveThreads, 2) k_lm_solve(BatchGrid g, Dev d0) {
+template <bool kLate>
+__global__ void __launch_bounds__(kLate ? kCrowdThreads : kSolveThreads, kLate ? kCrowdBlocksPerSM : kSolveBlocksPerSM)
+    k_lm_solve(BatchGrid g, Dev d0) {
   if (g.map == nullptr) {
-    lm_solve_impl(d0, grid_pos());
+    lm_solve_impl<kLate>(d0, grid_pos());
     return;
   }
   __shared__ Dev sd;
-  lm_solve_impl(sd, batch_block(g, sd));
+  lm_solve_impl<kLate>(sd, batch_block(g, sd));
 }
 
 // Energy of each candidate at the fixed association (normals and p~ held), then the accept step:
@@ -1424,12 +1450,8 @@ __global__ void __launch_bounds__(kBlock) k_lm_eval(BatchGrid g, Dev d0) {
   lm_eval_impl<c0, c1>(sd, batch_block(g, sd));
 }
 
-static int lm_solve_smem(int L) {
-  return (int)(lm_solve_table_offset(L) + ((sizeof(LinkTable) + 15) & ~(size_t)15) + (size_t)L * sizeof(DQ));
-}
-
 void launch_lm_solve(const Dev& d, cudaStream_t st) {
-  k_lm_solve<<<kCandidates, kSolveThreads, lm_solve_smem(d.L), st>>>(kSingle, d);
+  k_lm_solve<false><<<kCandidates, kSolveThreads, SolveLayout<false>::bytes(d.L), st>>>(kSingle, d);
 }
 
 void launch_lm_eval(const Dev& d, int /*phi_buf: the rows' records already hold x0 + phi*/, cudaStream_t st) {
@@ -1921,7 +1943,14 @@ void launch_normal_equations_b(const BatchGrid* gj, const int* nj, const BatchGr
 
 void launch_lm_b(const BatchGrid& glm, int nlm, const BatchGrid& gv, int nv, int max_links, int phi_buf,
                  cudaStream_t st) {
-  if (nlm > 0) k_lm_solve<<<nlm, kSolveThreads, lm_solve_smem(max_links), st>>>(glm, Dev{});
+  // 3 x 192 threads per SM where that takes fewer waves than 2 x 256: 64 sessions of 55 links 50 us against 70, 52
+  // sessions 48 against 66, 100 sessions (two waves either way) 80 against 72
+  auto waves = [nlm](int blocks_per_sm) { return (nlm + 152 * blocks_per_sm - 1) / (152 * blocks_per_sm); };
+  if (waves(kCrowdBlocksPerSM) < waves(kSolveBlocksPerSM)) {
+    k_lm_solve<true><<<nlm, kCrowdThreads, SolveLayout<true>::bytes(max_links), st>>>(glm, Dev{});
+  } else if (nlm > 0) {
+    k_lm_solve<false><<<nlm, kSolveThreads, SolveLayout<false>::bytes(max_links), st>>>(glm, Dev{});
+  }
   if (nv > 0) {
     const size_t sm = kCandidates * max_links * sizeof(DQ);
     k_lm_eval<0, kFirstPass><<<nv, kBlock, sm, st>>>(gv, Dev{});
@@ -1945,7 +1974,8 @@ int launch_shape_b(const BatchGrid& gv, int nv, int max_links, int sweeps, int s
 }
 
 static void configure_batched() {
-  cudaFuncSetAttribute(k_lm_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, lm_solve_smem(kMaxLinks));
+  cudaFuncSetAttribute(k_lm_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       SolveLayout<true>::bytes(kMaxLinks));
 }
 
 void configure_tc_kernels();
@@ -1960,7 +1990,8 @@ void configure_kernels() {
   cudaFuncSetAttribute(k_resid_jtj<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, jtj_smem_bytes(3, kMaxLinks));
   cudaFuncSetAttribute(k_resid_jtj<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, jtj_smem_bytes(4, kMaxLinks));
   cudaFuncSetAttribute(k_resid_jtj<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, jtj_smem_bytes(5, kMaxLinks));
-  cudaFuncSetAttribute(k_lm_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, lm_solve_smem(kMaxLinks));
+  cudaFuncSetAttribute(k_lm_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       SolveLayout<false>::bytes(kMaxLinks));
 }
 
 // Sets the kernels' shared-memory limits once per device (the attributes are per device).
