@@ -38,7 +38,7 @@ trk_status session_evict(trk_session* s);
 trk_status session_restore(trk_session* s);
 const trk_params& session_params(const trk_session* s);
 trk_status session_enqueue_frame(trk_session* s, const float* host_depth, cudaStream_t* stream_out);
-trk_status session_enqueue_results(trk_session* s, const ResultDst& dst);
+trk_status session_enqueue_results(trk_session* s, double* theta, float* phi4, double* energy, int* stats);
 void session_result_sizes(const trk_session* s, int* n_links, int* n_verts, int* n_energy);
 void session_forget_stream(trk_session* s, cudaStream_t st);
 }  // namespace trk
@@ -87,7 +87,7 @@ struct Staging {
   double* theta = nullptr;   // [L]
   double* energy = nullptr;  // [ne]
   int* stats = nullptr;      // [4]
-  float* phi = nullptr;      // [V][3]
+  float* phi = nullptr;      // [V][3] from a batched step, [V][4] from a session's own (Request::packed)
   const float* depth_dev = nullptr;  // device addresses of the same memory
   trk::ResultDst dst{};
 };
@@ -109,6 +109,7 @@ struct Request {
   clk::time_point t_submit, t_done;
   int state = 0;  // 0 queued, 1 on the GPU, 2 done
   trk_status status = TRK_OK;
+  bool packed = false;  // the offsets lie three floats a vertex
 };
 
 struct SessionSlot {
@@ -167,7 +168,7 @@ Staging* new_staging(size_t npx, int L, int V, int ne) {
   Staging* b = new Staging();
   const size_t o_th = up16(sizeof(float) * npx), o_en = o_th + up16(sizeof(double) * L),
                o_st = o_en + up16(sizeof(double) * std::max(ne, 1)), o_phi = o_st + 16,
-               total = o_phi + 3 * sizeof(float) * std::max(V, 1);
+               total = o_phi + sizeof(float4) * std::max(V, 1);
   if (cudaHostAlloc(&b->block, total, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
     delete b;
     return nullptr;
@@ -269,7 +270,7 @@ void launch_session(trk_server* sv, trk_session* s, SessionSlot& sl) {
   st->reqs.push_back(r);
   trk_status e = trk::session_enqueue_frame(s, r->b->depth, &st->st);
   if (e == TRK_OK)
-    e = trk::session_enqueue_results(s, r->b->dst);
+    e = trk::session_enqueue_results(s, r->b->theta, r->b->phi, r->b->energy, r->b->stats);
   if (e == TRK_OK && cudaLaunchHostFunc(st->st, on_step_done, st) != cudaSuccess) e = TRK_ERR_CUDA;
   if (e != TRK_OK) {
     fail_requests(sv, st->reqs, e);
@@ -288,6 +289,7 @@ void launch_batched(trk_server* sv, Step* slot, std::vector<trk_session*>& ss) {
     r->state = 1;
     sl.inflight = r;
     ++sv->inflight;
+    r->packed = true;
     slot->reqs.push_back(r);
     srcs.push_back(r->b->depth_dev);
     dst.push_back(r->b->dst);
@@ -608,7 +610,11 @@ trk_status trk_server_wait(trk_server* sv, uint64_t ticket, int64_t timeout_us, 
     trk::session_result_sizes(r->s, &L, &V, &ne);
     if (out->theta) std::memcpy(out->theta, b->theta, sizeof(double) * L);
     if (out->energy) std::memcpy(out->energy, b->energy, sizeof(double) * ne);
-    if (out->offsets) std::memcpy(out->offsets, b->phi, 3 * sizeof(float) * V);
+    if (out->offsets && r->packed) {
+      std::memcpy(out->offsets, b->phi, 3 * sizeof(float) * V);
+    } else if (out->offsets) {
+      for (int i = 0; i < V; ++i) std::memcpy(out->offsets + 3 * i, b->phi + 4 * i, 3 * sizeof(float));
+    }
     out->n_assoc_px = b->stats[0];
     out->n_assoc_verts = b->stats[1];
   }

@@ -249,8 +249,9 @@ struct trk_session {
   int device = 0;
   cudaStream_t stream = nullptr;
   cudaStream_t last_stream = nullptr;
-  cudaGraphExec_t graph = nullptr;       // a frame with the shape iterations
-  cudaGraphExec_t graph_pose = nullptr;  // a frame of pose iterations only (shape-match after frame 0, smooth-bind)
+  // the frame graphs: [0] pose iterations only (shape-match after frame 0, smooth-bind), [1] with the shape
+  // iterations; each without results, with them but for the offsets, with all (Results)
+  cudaGraphExec_t graph[2][3] = {};
   int frames_done = 0;                   // frames since the last trk_set_pose
   trk_params prm{};
   HostModel hm;
@@ -351,8 +352,26 @@ trk_status validate(const trk_mesh* m, const trk_skeleton* k, const trk_intrinsi
   return TRK_OK;
 }
 
-// Records the whole frame (pose iterations, then shape iterations) on st.
-void enqueue_frame(trk_session* s, cudaStream_t st, bool with_shape) {
+enum Results { kNoResults = 0, kWithoutOffsets = 1, kWithOffsets = 2 };
+
+// The current results into the session's pinned staging, by one kernel (a copy each costs more than the copying).
+//
+// The kernel is launched where its stream is idle or belongs to a frame's graph, never behind a graph that runs: streams share a
+// few hardware queues, and a launch that waits for its stream's graph holds up the graphs of other streams
+// behind it (64 threads that each track a session of 5k vertices: 8,200 frames/s, in the graph 11,400; 50k:
+// 3,600 and 3,970).
+void enqueue_results(trk_session* s, Results what, cudaStream_t st) {
+  if (what == kNoResults) return;
+  ResultDst dst{};
+  dst.theta = s->h_pinned;  // [L] theta, [ne] energy, [4] stats
+  dst.energy = dst.theta + s->d.L;
+  dst.stats = reinterpret_cast<int*>(dst.energy + s->prm.pose_iters + s->prm.shape_iters);
+  dst.phi = what == kWithOffsets ? s->h_phi : nullptr;
+  launch_results(s->d, dst, st);
+}
+
+// Records the whole frame (pose iterations, then shape iterations) and its results on st.
+void enqueue_frame(trk_session* s, cudaStream_t st, bool with_shape, Results results) {
   const Dev& d = s->d;
   const int P = s->prm.pose_iters, S = with_shape ? s->prm.shape_iters : 0;
   int cur = 0;
@@ -376,6 +395,7 @@ void enqueue_frame(trk_session* s, cudaStream_t st, bool with_shape) {
     cur = launch_shape(d, cur, P + it, st);
   }
   if (cur != 0) cudaMemcpyAsync(d.phi[0], d.phi[cur], sizeof(float4) * d.V, cudaMemcpyDeviceToDevice, st);
+  enqueue_results(s, results, st);
 }
 
 // Whether the next frame runs the shape iterations: always in tracking mode, on the first frame after
@@ -384,14 +404,22 @@ bool next_frame_with_shape(const trk_session* s) {
   return s->prm.mode == TRK_MODE_TRACK || (s->prm.mode == TRK_MODE_SHAPE_MATCH && s->frames_done == 0);
 }
 
+void destroy_graphs(trk_session* s) {
+  for (auto& g : s->graph)
+    for (cudaGraphExec_t& e : g) {
+      if (e) cudaGraphExecDestroy(e);
+      e = nullptr;
+    }
+}
+
 // The frame graph for the next frame (captured on first use).
-trk_status frame_graph(trk_session* s, cudaGraphExec_t* out) {
+trk_status frame_graph(trk_session* s, Results results, cudaGraphExec_t* out) {
   const bool with_shape = next_frame_with_shape(s);
-  cudaGraphExec_t& ge = with_shape ? s->graph : s->graph_pose;
+  cudaGraphExec_t& ge = s->graph[with_shape][results];
   if (!ge) {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
-    enqueue_frame(s, s->stream, with_shape);
+    enqueue_frame(s, s->stream, with_shape, results);
     CK(cudaStreamEndCapture(s->stream, &g));
     cudaError_t e = cudaGraphInstantiate(&ge, g, 0);
     cudaGraphDestroy(g);
@@ -401,30 +429,25 @@ trk_status frame_graph(trk_session* s, cudaGraphExec_t* out) {
   return TRK_OK;
 }
 
-trk_status fetch_result(trk_session* s, cudaStream_t st, trk_result* out) {
-  if (!out) return TRK_OK;
-  const Dev& d = s->d;
-  const int ne = s->prm.pose_iters + s->prm.shape_iters;
-  double* h = s->h_pinned;  // [L] theta, [ne] energy, [1] stats
-  // one kernel writes them straight into the pinned memory (a copy each cost more than the copying)
-  ResultDst dst{};
-  dst.theta = h;
-  dst.energy = h + d.L;
-  dst.stats = reinterpret_cast<int*>(h + d.L + ne);
-  dst.phi = out->offsets ? s->h_phi : nullptr;
-  launch_results(d, dst, st);
+// The results in the pinned staging, once st has got to them, into out.
+trk_status take_results(trk_session* s, cudaStream_t st, trk_result* out) {
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
-  if (out->theta) std::memcpy(out->theta, h, sizeof(double) * d.L);
-  if (out->energy) std::memcpy(out->energy, h + d.L, sizeof(double) * ne);
+  if (!out) return TRK_OK;
+  const int L = s->d.L, ne = s->prm.pose_iters + s->prm.shape_iters;
+  const double* h = s->h_pinned;
+  if (out->theta) std::memcpy(out->theta, h, sizeof(double) * L);
+  if (out->energy) std::memcpy(out->energy, h + L, sizeof(double) * ne);
   int stats[4];
-  std::memcpy(stats, h + d.L + ne, sizeof(stats));
+  std::memcpy(stats, h + L + ne, sizeof(stats));
   out->n_assoc_px = stats[0];
   out->n_assoc_verts = stats[1];
   if (stats[3]) return fail(TRK_ERR_TIMEOUT, "a tensor-core completion wait ran out; results are not valid");
-  if (out->offsets) std::memcpy(out->offsets, s->h_phi, 3 * sizeof(float) * d.V);
+  if (out->offsets) std::memcpy(out->offsets, s->h_phi, 3 * sizeof(float) * s->d.V);
   return TRK_OK;
 }
+
+Results wanted(const trk_result* out) { return !out ? kNoResults : out->offsets ? kWithOffsets : kWithoutOffsets; }
 
 trk_status sync_check(trk_session* s) {
   CK(cudaGetLastError());
@@ -457,7 +480,7 @@ void session_result_sizes(const trk_session* s, int* n_links, int* n_verts, int*
 // H2D of the frame's depth and the frame graph, on the session's stream
 trk_status session_enqueue_frame(trk_session* s, const float* host_depth, cudaStream_t* stream_out) {
   cudaGraphExec_t ge;
-  TRY(frame_graph(s, &ge));
+  TRY(frame_graph(s, kNoResults, &ge));
   CK(cudaMemcpyAsync(const_cast<float*>(s->d.depth), host_depth, sizeof(float) * s->d.cam.W * s->d.cam.H,
                      cudaMemcpyHostToDevice, s->stream));
   launch_tiles(s->d, s->d.depth, s->stream);  // the frame's occupied tiles (the graph's association reads them)
@@ -467,10 +490,16 @@ trk_status session_enqueue_frame(trk_session* s, const float* host_depth, cudaSt
   *stream_out = s->stream;
   return TRK_OK;
 }
-// The frame's results into (pinned) host buffers, on the session's stream
-trk_status session_enqueue_results(trk_session* s, const ResultDst& dst) {
-  launch_results(s->d, dst, s->stream);
-  CK(cudaGetLastError());
+// The frame's results into pinned host buffers, on the session's stream: copies (the offsets as they lie, four floats a
+// vertex), which wait behind the frame's graph without holding up other streams' (enqueue_results).  64 streams of 50k
+// vertices: 3,970 frames/s, with the kernel 3,780; of packing on the device and copying, 3,780 too.
+trk_status session_enqueue_results(trk_session* s, double* theta, float* phi4, double* energy, int* stats) {
+  const Dev& d = s->d;
+  const int ne = s->prm.pose_iters + s->prm.shape_iters;
+  CK(cudaMemcpyAsync(theta, d.theta, sizeof(double) * d.L, cudaMemcpyDeviceToHost, s->stream));
+  CK(cudaMemcpyAsync(phi4, d.phi[0], sizeof(float4) * d.V, cudaMemcpyDeviceToHost, s->stream));
+  if (ne > 0) CK(cudaMemcpyAsync(energy, d.energy, sizeof(double) * ne, cudaMemcpyDeviceToHost, s->stream));
+  CK(cudaMemcpyAsync(stats, d.stats, sizeof(int) * 4, cudaMemcpyDeviceToHost, s->stream));
   return TRK_OK;
 }
 }  // namespace trk
@@ -486,8 +515,7 @@ void trk_destroy(trk_session* s) {
   cudaSetDevice(s->device);
   if (s->last_stream && s->last_stream != s->stream) cudaStreamSynchronize(s->last_stream);
   if (s->stream) cudaStreamSynchronize(s->stream);
-  if (s->graph) cudaGraphExecDestroy(s->graph);
-  if (s->graph_pose) cudaGraphExecDestroy(s->graph_pose);
+  destroy_graphs(s);
   if (s->arena) vmm_free(&s->block);  // the streams above are idle
   if (s->h_pinned) cudaFreeHost(s->h_pinned);
   if (s->h_phi) cudaFreeHost(s->h_phi);
@@ -629,9 +657,7 @@ trk_status evict(trk_session* s) {
   CK(cudaMemcpyAsync(&s->ev_lam, d.lam, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
   CK(cudaMemcpyAsync(s->ev_phi.data(), d.phi[0], sizeof(float4) * d.V, cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
-  if (s->graph) cudaGraphExecDestroy(s->graph);
-  if (s->graph_pose) cudaGraphExecDestroy(s->graph_pose);
-  s->graph = s->graph_pose = nullptr;
+  destroy_graphs(s);
   vmm_free(&s->block);  // the memory is back on the device when the eviction returns
   s->arena = nullptr;
   carve_all(s);  // every device pointer back to NULL
@@ -1060,7 +1086,7 @@ trk_status trk_track_frame(trk_session* s, const float* depth_m, trk_result* out
   if (!s || !depth_m) return fail(TRK_ERR_INVALID_ARG, "NULL argument");
   NEED_RESIDENT(s);
   cudaGraphExec_t ge;
-  TRY(frame_graph(s, &ge));
+  TRY(frame_graph(s, wanted(out), &ge));
   const Dev& d = s->d;
   CK(cudaMemcpyAsync(const_cast<float*>(d.depth), depth_m, sizeof(float) * d.cam.W * d.cam.H, cudaMemcpyHostToDevice,
                      s->stream));
@@ -1068,8 +1094,7 @@ trk_status trk_track_frame(trk_session* s, const float* depth_m, trk_result* out
   CK(cudaGraphLaunch(ge, s->stream));
   ++s->frames_done;
   s->last_stream = s->stream;
-  TRY(fetch_result(s, s->stream, out));
-  return sync_check(s);
+  return take_results(s, s->stream, out);
 }
 
 trk_status trk_track_frame_device(trk_session* s, const float* d_depth_m, void* cuda_stream) {
@@ -1077,7 +1102,7 @@ trk_status trk_track_frame_device(trk_session* s, const float* d_depth_m, void* 
   if (!s || !d_depth_m) return fail(TRK_ERR_INVALID_ARG, "NULL argument");
   NEED_RESIDENT(s);
   cudaGraphExec_t ge;
-  TRY(frame_graph(s, &ge));
+  TRY(frame_graph(s, kNoResults, &ge));
   cudaStream_t st = cuda_stream ? (cudaStream_t)cuda_stream : s->stream;
   launch_tiles(s->d, d_depth_m, st);  // copies the caller's depth and lists its occupied tiles: no memcpy
   CK(cudaGraphLaunch(ge, st));
@@ -1091,8 +1116,9 @@ trk_status trk_read_result(trk_session* s, trk_result* out) {
   if (!s) return fail(TRK_ERR_INVALID_ARG, "NULL argument");
   NEED_RESIDENT(s);
   cudaStream_t st = s->last_stream ? s->last_stream : s->stream;
-  TRY(fetch_result(s, st, out));
-  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(st));  // (enqueue_results)
+  enqueue_results(s, wanted(out), st);
+  TRY(take_results(s, st, out));
   s->last_stream = nullptr;  // the frame is done: nothing left to wait for on that stream
   return TRK_OK;
 }
