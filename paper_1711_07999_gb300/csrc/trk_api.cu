@@ -466,7 +466,8 @@ trk_status session_evict(trk_session* s) { return evict(s); }
 trk_status session_restore(trk_session* s) { return materialize(s); }
 const Dev& session_dev(const trk_session* s) { return s->d; }
 const trk_params& session_params(const trk_session* s) { return s->prm; }
-void session_set_last_stream(trk_session* s, cudaStream_t st) { s->last_stream = st; }
+// (a batch's NULL is the legacy default stream; here NULL means that there is no frame to wait for)
+void session_set_last_stream(trk_session* s, cudaStream_t st) { s->last_stream = st ? st : cudaStreamLegacy; }
 // The owner of stream st has waited for it and is about to destroy it: the session's last frame there is done.
 void session_forget_stream(trk_session* s, cudaStream_t st) {
   if (s->last_stream == st) s->last_stream = nullptr;
