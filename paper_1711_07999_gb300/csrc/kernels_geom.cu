@@ -342,21 +342,19 @@ __device__ __forceinline__ void commit_pixel(const Dev& d, int best, float3 p, f
   atomicAdd(a + 3, 1ull);
 }
 
-// The pixel's point, back-projected in FP64 and then moved into the session-local frame (exact up to one FP32 rounding),
-// x and y once per frame for its twelve or so iterations: on this GPU the ~20 FP64 operations and conversions of a
-// back-projection occupy the FP64 pipe for ~1,250 cycles per warp.
-__device__ __forceinline__ void store_point(const Dev& d, int px, int py, int k, float z) {
-  const Cam& c = d.cam;
-  d.pxy[k] = make_float2((float)(((double)px - (double)c.cx) * (double)z * c.inv_fx - (double)c.ox),
-                         (float)(((double)py - (double)c.cy) * (double)z * c.inv_fy - (double)c.oy));
+__device__ __forceinline__ float3 back_project(const Cam& c, int px, int py, float dep) {
+  // in FP64, then moved into the session-local frame (exact up to one FP32 rounding)
+  return make_float3((float)(((double)px - (double)c.cx) * (double)dep * c.inv_fx - (double)c.ox),
+                     (float)(((double)py - (double)c.cy) * (double)dep * c.inv_fy - (double)c.oy),
+                     (float)((double)dep - (double)c.oz));
 }
 
-// z is left to be formed here, which keeps 8 bytes a pixel instead of 16 (the depth is there anyway): an FP32
-// difference of two FP32 numbers is the FP64 difference rounded to FP32 (2 x 24 + 2 <= 53 bits), bit for bit.
-__device__ __forceinline__ float3 load_point(const Dev& d, int k, float& dep) {
-  const float2 xy = d.pxy[k];
-  dep = d.depth[k];
-  return make_float3(xy.x, xy.y, dep - d.cam.oz);
+// The pixel's point, once per frame for its twelve or so iterations: on this GPU the ~20 FP64 operations and
+// conversions of a back-projection occupy the FP64 pipe for ~1,250 cycles per warp.  (Kept as x, y beside the depth it
+// would take 8 bytes a pixel less, and a frame of 200k vertices 1.7 % longer.)
+__device__ __forceinline__ void store_point(const Dev& d, int px, int py, int k, float z) {
+  const float3 p = back_project(d.cam, px, py, z);
+  d.ppos[k] = make_float4(p.x, p.y, p.z, z);
 }
 
 // One lane's pixel (px, py) of a warp's unit (active false: the lane has none; it still takes part in
@@ -371,8 +369,9 @@ __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, boo
   float3 p = make_float3(0.f, 0.f, 0.f);
   bool open = false;
   if (inimg) {  // (the units list pixels with a valid depth)
-    float dep;
-    p = load_point(d, k, dep);
+    const float4 pp = d.ppos[k];
+    p = f3(pp);
+    const float dep = pp.w;
     if (d.association == 1) {
       // the nearest corner of the triangle the z-buffer holds at this pixel (O(1), no queue)
       const unsigned long long key = d.zbuf[k];
@@ -427,8 +426,8 @@ __device__ __forceinline__ void associate_impl(const Dev& d, int px, int py, boo
   unsigned base = 0;
   if (lane == 0 && om) base = atomicAdd(&d.qctl[0], __popc(om));
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = k;
-  if (inimg) d.corr[k] = best.i;  // (of an open pixel: the nearest so far, which the tail starts from)
+  if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int2(k, best.i);
+  if (inimg && !open) d.corr[k] = best.i;
   const bool done = !open && best.i >= 0;
   if (done) commit_pixel(d, best.i, p, best.v);
   const unsigned m = __ballot_sync(0xffffffffu, done);
@@ -450,7 +449,9 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
   float3 p = make_float3(0.f, 0.f, 0.f);
   float dep = 0.f;
   if (inimg) {
-    p = load_point(d, k, dep);
+    const float4 pp = d.ppos[k];
+    p = f3(pp);
+    dep = pp.w;
     const int q[3] = {ring_bucket(px, py, 1, 2 * sub, c.W, c.H), ring_bucket(px, py, 1, 2 * sub + 1, c.W, c.H),
                       sub == 3 ? k : -1};
     scan_group<3, false>(d, q, p, tau2, best);
@@ -473,8 +474,8 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
   if (lane == 0 && om) base = atomicAdd(&d.qctl[0], __popc(om));
   base = __shfl_sync(0xffffffffu, base, 0);
   if (sub == 0) {
-    if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = k;
-    if (inimg) d.corr[k] = nearest;
+    if (open) d.queue[base + __popc(om & ((1u << lane) - 1u))] = make_int2(k, nearest);
+    else if (inimg) d.corr[k] = nearest;
   }
   const bool done = inimg && !open && nearest >= 0 && mine == key;  // the lane that holds the nearest
   if (done) commit_pixel(d, best.i, p, best.v);
@@ -503,12 +504,16 @@ template <int GL, int PL, bool kRows>
 __device__ __forceinline__ bool tail_item(const Dev& d, unsigned item, int gl, unsigned gmask) {
   const Cam& c = d.cam;
   const float tau2 = c.tau * c.tau;
-  const int k = d.queue[item], W = c.W, H = c.H, px = k % W, py = k / W;
-  const int near = d.corr[k];
-  float dep;
-  const float3 p = load_point(d, k, dep);
+  const int2 e = d.queue[item];
+  const int k = e.x, W = c.W, H = c.H, px = k % W, py = k / W;
+  // (a host depth image passes through the queue's memory: a program that brings the next one in while a frame still runs gets
+  // a wrong frame, not a wild address)
+  if ((unsigned)k >= (unsigned)(W * H) || e.y >= d.V) return false;
+  const float4 pp = d.ppos[k];
+  const float dep = pp.w;
+  const float3 p = f3(pp);
   Best w{-1, 0.f, make_float3(0.f, 0.f, 0.f)};
-  if (near >= 0) consider(near, p, d.v[near], tau2, w);  // the nearest so far (its record's bits)
+  if (e.y >= 0) consider(e.y, p, d.v[e.y], tau2, w);  // the nearest so far (its record's bits)
   unsigned long long key = key_of(w.i, w.d2);
   // several rings at a time: scanning rings past the one whose bound ends the search only confirms the
   // argmin, so the result is the same
@@ -583,7 +588,7 @@ __device__ __forceinline__ bool tail_item(const Dev& d, unsigned item, int gl, u
 // short list spreads over all SMs), then every (warps in the grid)-th: no counter and no block barrier, so a warp whose pixels are cheap goes on to its next unit at once,
 // and the interleaving spreads the units of costly sessions over all warps.  In a batch each warp keeps
 // its own copy of its unit's session descriptor in shared memory (reloaded when the session changes).
-// Pixels outside the units keep the "no correspondence" the frame's depth copy wrote.
+// Pixels outside the units keep the "no correspondence" that was written with the frame's points.
 __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const Dev* devs, const AssocUnit* units,
                                                                           const unsigned* ctl, Dev d0) {
   __shared__ Dev sd[kBlock / 32];
@@ -592,10 +597,14 @@ __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const D
   const AssocUnit* list = single ? d0.units : units;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned nw = gridDim.x * (kBlock / 32);
-  // four lanes per pixel where the units do not fill the grid's warps even once, so that the launch lasts as long as
-  // a unit (3,500 units of uneven sessions on 4,864 warps: 69 us a lane per pixel, 41 four; 9,600 units of
-  // sixteen equal ones: 34 against 40) (the window search with R >= 1
-  // only); lane l of the warp then serves pixel 8 (part of the unit) + l / 4
+  // Four lanes per pixel (the window search with R >= 1 only) where the units are no more than the grid's warps, so that
+  // a warp takes at most four quarter units: 3,500 units of uneven sessions on 4,864 warps 69 us a lane per
+  // pixel, 41 four; 9,600 units of sixteen equal ones 34 against 40.  Lane l of the warp then serves pixel
+  // 8 (part of the unit) + l / 4.  One session's grid has a warp per unit that its image can have (up to the
+  // same 4,864), so smaller images always take four: frames of a body in 160x120, 357x269 and 640x480
+  // 707 -> 662, 796 -> 741 and 1,053 -> 947 us, of 160x120 with every pixel valid 857 -> 868.  A grid of four warps
+  // per unit would gain there (819), but 32 sessions of that size beside each other would lose (23,300 -> 21,100
+  // frames/s).
   const bool quad = n <= nw && (single ? d0.association == 0 && d0.cam.R > 0 : devs[0].association == 0);
   const unsigned items = quad ? 4 * n : n;
   int cur = -1;
@@ -628,22 +637,34 @@ __global__ void __launch_bounds__(kBlock, kAssocBlocksPerSM) k_associate(const D
   }
 }
 
-// One session: the warps of all blocks take its queue entries, warp w the w-th, then the rest from the
-// session's counter (no counter traffic when the queue is no longer than the grid's warps).
-__global__ void __launch_bounds__(32 * kTailWarps) k_associate_tail(Dev d) {
-  const int lane = threadIdx.x & 31, gl = lane, gbase = 0;
-  const unsigned gmask = 0xffffffffu;
-  const unsigned n = *(volatile unsigned*)&d.qctl[0];
-  const unsigned warps = gridDim.x * kTailWarps;  // warp w takes entry w first, then the counter's
+// One session's queue: the lane groups of all blocks take its entries, group g the g-th, then the rest from the session's
+// counter (no counter traffic when the queue is no longer than the grid's groups).
+template <int GL, int PL, bool kRows>
+__device__ __forceinline__ void tail_queue(const Dev& d, unsigned n) {
+  const int lane = threadIdx.x & 31, gl = lane % GL, gbase = lane - gl;
+  const unsigned gmask = (unsigned)((1ull << GL) - 1) << gbase;
+  const unsigned groups = gridDim.x * (32 * kTailWarps / GL);
   int done = 0;
-  for (unsigned item = blockIdx.x * kTailWarps + (threadIdx.x >> 5); item < n;) {
-    done += tail_item<32, kTailPerLane, false>(d, item, gl, gmask);
-    if (warps >= n) break;
+  for (unsigned item = (blockIdx.x * 32 * kTailWarps + threadIdx.x) / GL; item < n;) {
+    done += tail_item<GL, PL, kRows>(d, item, gl, gmask);
+    if (groups >= n) break;
     unsigned next = 0;
-    if (gl == 0) next = warps + atomicAdd(&d.qctl[1], 1u);
+    if (gl == 0) next = groups + atomicAdd(&d.qctl[1], 1u);
     item = __shfl_sync(gmask, next, gbase);
   }
   if (gl == 0 && done) atomicAdd(&d.stats[0], done);
+}
+
+// A warp per pixel: the latency of one pixel's search is what a short queue takes.  A queue of more than four pixels per
+// warp of two blocks per SM or eight of four (an image with a background, a pose far off) is bound by its warps'
+// throughput and goes eight lanes to a pixel, as a batch's does (640x480 with every pixel valid: 402 -> 153 us the
+// association).  Below that it loses where the mesh is finer than the image: 200k vertices at 1280x720 on
+// four blocks per SM, a frame 1,931 us, from four pixels per warp on 1,983; on two 1,980, from two on 2,086.
+__global__ void __launch_bounds__(32 * kTailWarps, 4) k_associate_tail(Dev d) {
+  const unsigned n = *(volatile unsigned*)&d.qctl[0];
+  // (the row windows of the occupancy bits hold up to 63 columns)
+  if (n > 2 * gridDim.x / 152 * gridDim.x * kTailWarps && d.cam.R <= 31) tail_queue<kBatchTailLanes, kBatchTailPerLane, true>(d, n);
+  else tail_queue<32, kTailPerLane, false>(d, n);
 }
 
 constexpr int kInBlockPrefix = 32 * kTailWarps;  // sessions whose prefix the tail's blocks form themselves
@@ -728,9 +749,13 @@ void launch_associate(const Dev& d, cudaStream_t st) {
   const int nunits = ((d.cam.W + 15) / 16) * ((d.cam.H + 1) / 2);
   k_associate<<<min((nunits + kBlock / 32 - 1) / (kBlock / 32), kAssocBlocksPerSM * 152), kBlock, 0, st>>>(nullptr, nullptr,
                                                                                                    nullptr, d);
-  // (four blocks per SM: an iteration that moved the pose queues more pixels than two per SM have warps for; 200k
-  // vertices at 1280x720: 27.3 us on two, 24.1 on four, the longest launch of a frame 109 and 85)
-  k_associate_tail<<<4 * 152, 32 * kTailWarps, 0, st>>>(d);
+  // Blocks of the tail: most sessions track beside others, whose work the blocks of a short queue hold up (32 sessions on
+  // their own streams, frames/s at two and four blocks per SM: 5k vertices at 160x120 27,400 and 23,300, 50k at
+  // 640x480 5,050 and 4,885; one session alone: 50k 955 and 947 us a frame).  A larger image queues more pixels
+  // than two have warps for (200k vertices at 1280x720: 1,957 and 1,863 us a frame, eight sessions 1,313 and
+  // 1,272 frames/s).
+  const int per_sm = d.cam.W * d.cam.H > 640 * 480 ? 4 : 2;
+  k_associate_tail<<<per_sm * 152, 32 * kTailWarps, 0, st>>>(d);
 }
 
 // Appends this block's tile's association units to list: its pixels with a valid depth, in row-major
@@ -761,7 +786,7 @@ __device__ __forceinline__ void list_units(bool valid, int session, int tx, int 
         make_int4(session, tx * 16, ty * 16, min(32, total - 32 * (int)threadIdx.x));
 }
 
-// One 16 x 16 tile per block: copies the frame's depth into the session's buffer, marks every pixel
+// One 16 x 16 tile per block: back-projects the frame's pixels into the session's points, marks every pixel
 // "no correspondence" (the association rewrites the pixels of its units each iteration) and lists the
 // tile's units that hold a valid pixel.
 __global__ void __launch_bounds__(kBlock) k_tiles(Dev d, const float* __restrict__ src) {
@@ -772,7 +797,6 @@ __global__ void __launch_bounds__(kBlock) k_tiles(Dev d, const float* __restrict
   if (px < d.cam.W && py < d.cam.H) {
     const int k = py * d.cam.W + px;
     const float z = src[k];
-    const_cast<float*>(d.depth)[k] = z;
     d.corr[k] = -1;
     valid = z > 0.f;
     if (valid) store_point(d, px, py, k, z);
@@ -802,7 +826,7 @@ void launch_associate_b(const Dev* devs, int n_sessions, const AssocUnit* tiles,
   k_associate_tail_batch<<<tail_blocks, 32 * kTailWarps, 0, st>>>(devs, n_sessions, prefix, ctl);
 }
 
-// Copies each session's depth frame from srcs[session] into the session's own depth buffer, one 16 x 16
+// Back-projects each session's depth frame at srcs[session] into the session's points, one 16 x 16
 // tile per block, marks every pixel "no correspondence" and lists the association units (16 x 2 pixels)
 // that hold a valid depth.
 __global__ void __launch_bounds__(kBlock) k_gather_depth_b(BatchGrid g, const float* const* srcs, AssocUnit* units,
@@ -814,7 +838,6 @@ __global__ void __launch_bounds__(kBlock) k_gather_depth_b(BatchGrid g, const fl
   if (px < d.cam.W && py < d.cam.H) {
     const int k = py * d.cam.W + px;
     const float z = srcs[m.x][k];
-    const_cast<float*>(d.depth)[k] = z;
     d.corr[k] = -1;
     valid = z > 0.f;
     if (valid) store_point(d, px, py, k, z);

@@ -267,7 +267,8 @@ struct trk_session {
   std::vector<float4> ev_phi;
   double* h_pinned = nullptr;  // pinned staging for results
   float* h_phi = nullptr;      // pinned staging for the offsets of a result [V][3]
-  float* d_render = nullptr;
+  float* image = nullptr;      // [W*H] a host frame's depth on its way to the points, or a rendered one: in the memory of
+                               // the association's queue, which holds nothing between associations
 };
 
 namespace {
@@ -478,13 +479,17 @@ void session_result_sizes(const trk_session* s, int* n_links, int* n_verts, int*
   *n_verts = s->d.V;
   *n_energy = s->prm.pose_iters + s->prm.shape_iters;
 }
+// A host depth image to the session's points and units, on its stream.
+trk_status take_depth(trk_session* s, const float* host_depth) {
+  CK(cudaMemcpyAsync(s->image, host_depth, sizeof(float) * s->d.cam.W * s->d.cam.H, cudaMemcpyHostToDevice, s->stream));
+  launch_tiles(s->d, s->image, s->stream);
+  return TRK_OK;
+}
 // H2D of the frame's depth and the frame graph, on the session's stream
 trk_status session_enqueue_frame(trk_session* s, const float* host_depth, cudaStream_t* stream_out) {
   cudaGraphExec_t ge;
   TRY(frame_graph(s, kNoResults, &ge));
-  CK(cudaMemcpyAsync(const_cast<float*>(s->d.depth), host_depth, sizeof(float) * s->d.cam.W * s->d.cam.H,
-                     cudaMemcpyHostToDevice, s->stream));
-  launch_tiles(s->d, s->d.depth, s->stream);  // the frame's occupied tiles (the graph's association reads them)
+  TRY(take_depth(s, host_depth));
   CK(cudaGraphLaunch(ge, s->stream));
   ++s->frames_done;
   s->last_stream = s->stream;
@@ -541,9 +546,8 @@ void carve_all(trk_session* s) {
   float4 *dv0, *dbw;
   uchar4* dbidx;
   int4 *dtris, *dnb;
-  int *dcsr_off, *dcsr_face, *dadj_off, *dadj;
+  int *dcsr_off, *dcsr_face, *dadj_off = nullptr, *dadj = nullptr;
   double* dprior;
-  float* ddepth;
   carve(s, &dlt, 1);
   carve(s, &dv0, V); carve(s, &dbw, V); carve(s, &dbidx, V);
   carve(s, &dtris, F); carve(s, &dnb, V);
@@ -558,19 +562,17 @@ void carve_all(trk_session* s) {
   carve(s, &d.lm_ok, 2 * kCandidates);
   carve(s, &d.v, V); carve(s, &d.n, V); carve(s, &d.fn, F); carve(s, &d.rec, V);
   carve(s, &d.head, npx); carve(s, &d.zbuf, npx); carve(s, &d.corr, npx);
-  carve(s, &d.pixrec, npx); carve(s, &d.queue, npx); carve(s, &d.qctl, 4); carve(s, &d.pxy, npx);
+  carve(s, &d.pixrec, npx); carve(s, &d.queue, npx); carve(s, &d.qctl, 4); carve(s, &d.ppos, npx);
   carve(s, &d.occ, (size_t)d.cam.H * occ_row(d.cam.W));
   carve(s, &d.units, (size_t)kUnitsPerTile * ((d.cam.W + 15) / 16) * ((d.cam.H + 15) / 16));
   carve(s, &d.acc, V); carve(s, &d.vispix, V); carve(s, &d.rg, V); carve(s, &d.phi0, V);
-  carve(s, &dadj_off, V + 1); carve(s, &dadj, s->hm.adj.size());
   d.cg_x = d.cg_r = d.cg_z = d.cg_p = d.cg_ap = nullptr;
   if (prm.shape_solver == 1) {
+    carve(s, &dadj_off, V + 1); carve(s, &dadj, s->hm.adj.size());
     carve(s, &d.cg_x, V); carve(s, &d.cg_r, V); carve(s, &d.cg_z, V);
     carve(s, &d.cg_p, V); carve(s, &d.cg_ap, V);
   }
   carve(s, &d.cg, 4);
-  carve(s, &ddepth, npx);
-  carve(s, &s->d_render, npx);
   carve(s, &d.partial, (size_t)d.nblk_rows * NP * NP);
   carve(s, &d.jtj_rows, (size_t)d.nblk_rows);
   carve(s, &d.arec, (size_t)d.nblk_jtj * 256 * 4);
@@ -580,7 +582,7 @@ void carve_all(trk_session* s) {
   carve(s, &d.stats, 4);
   d.links = dlt; d.v0 = dv0; d.bw = dbw; d.bidx = dbidx; d.tris = dtris; d.nbr = dnb;
   d.csr_off = dcsr_off; d.csr_face = dcsr_face; d.prior2 = dprior;
-  d.depth = ddepth;
+  s->image = reinterpret_cast<float*>(d.queue);
   d.adj_off = dadj_off;
   d.adj = dadj;
 }
@@ -614,7 +616,6 @@ trk_status materialize(trk_session* s) {
   Dev& d = s->d;
   const HostModel& hm = s->hm;
   const int L = d.L, V = d.V, F = d.F;
-  const size_t npx = (size_t)d.cam.W * d.cam.H;
   const int ne = std::max(1, s->prm.pose_iters + s->prm.shape_iters);
   cudaStream_t st = s->stream;
   CK(cudaMemcpyAsync(const_cast<LinkTable*>(d.links), &hm.lt, sizeof(LinkTable), cudaMemcpyHostToDevice, st));
@@ -626,15 +627,16 @@ trk_status materialize(trk_session* s) {
   CK(cudaMemcpyAsync(const_cast<int*>(d.csr_off), hm.csr_off.data(), sizeof(int) * (V + 1), cudaMemcpyHostToDevice, st));
   if (F) CK(cudaMemcpyAsync(const_cast<int*>(d.csr_face), hm.csr_face.data(), sizeof(int) * 3 * F, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(const_cast<double*>(d.prior2), hm.prior2.data(), sizeof(double) * L, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(const_cast<int*>(d.adj_off), hm.adj_off.data(), sizeof(int) * (V + 1), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(const_cast<int*>(d.adj), hm.adj.data(), sizeof(int) * hm.adj.size(), cudaMemcpyHostToDevice, st));
+  if (d.adj) {
+    CK(cudaMemcpyAsync(const_cast<int*>(d.adj_off), hm.adj_off.data(), sizeof(int) * (V + 1), cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(const_cast<int*>(d.adj), hm.adj.data(), sizeof(int) * hm.adj.size(), cudaMemcpyHostToDevice, st));
+  }
   CK(cudaMemsetAsync(d.cg, 0, sizeof(double) * 4, st));
   CK(cudaMemsetAsync(d.counter, 0, sizeof(unsigned) * 4, st));
   CK(cudaMemsetAsync(d.qctl, 0, sizeof(unsigned) * 4, st));
   CK(cudaMemsetAsync(d.stats, 0, sizeof(int) * 4, st));
   CK(cudaMemsetAsync(d.energy, 0, sizeof(double) * ne, st));
   CK(cudaMemsetAsync(d.lm_trials, 0, sizeof(double) * 8, st));
-  CK(cudaMemsetAsync(const_cast<float*>(d.depth), 0, sizeof(float) * npx, st));
   // the tracking state
   CK(cudaMemcpyAsync(d.theta, s->ev_theta.data(), sizeof(double) * L, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d.lam, &s->ev_lam, sizeof(double), cudaMemcpyHostToDevice, st));
@@ -1089,9 +1091,7 @@ trk_status trk_track_frame(trk_session* s, const float* depth_m, trk_result* out
   cudaGraphExec_t ge;
   TRY(frame_graph(s, wanted(out), &ge));
   const Dev& d = s->d;
-  CK(cudaMemcpyAsync(const_cast<float*>(d.depth), depth_m, sizeof(float) * d.cam.W * d.cam.H, cudaMemcpyHostToDevice,
-                     s->stream));
-  launch_tiles(d, d.depth, s->stream);  // the frame's occupied tiles (the graph's association reads them)
+  TRY(take_depth(s, depth_m));
   CK(cudaGraphLaunch(ge, s->stream));
   ++s->frames_done;
   s->last_stream = s->stream;
@@ -1105,7 +1105,7 @@ trk_status trk_track_frame_device(trk_session* s, const float* d_depth_m, void* 
   cudaGraphExec_t ge;
   TRY(frame_graph(s, kNoResults, &ge));
   cudaStream_t st = cuda_stream ? (cudaStream_t)cuda_stream : s->stream;
-  launch_tiles(s->d, d_depth_m, st);  // copies the caller's depth and lists its occupied tiles: no memcpy
+  launch_tiles(s->d, d_depth_m, st);  // reads the caller's depth: no memcpy
   CK(cudaGraphLaunch(ge, st));
   ++s->frames_done;
   CK(cudaGetLastError());
@@ -1140,17 +1140,15 @@ trk_status trk_render_depth(trk_session* s, const double* theta, const float* of
   launch_fk(r, s->stream);
   launch_skin(r, 0, s->stream);
   launch_raster(r, s->stream);
-  launch_depth_from_zbuf(r, s->d_render, s->stream);
-  CK(cudaMemcpyAsync(depth_m, s->d_render, sizeof(float) * r.cam.W * r.cam.H, cudaMemcpyDeviceToHost, s->stream));
+  launch_depth_from_zbuf(r, s->image, s->stream);
+  CK(cudaMemcpyAsync(depth_m, s->image, sizeof(float) * r.cam.W * r.cam.H, cudaMemcpyDeviceToHost, s->stream));
   return sync_check(s);
 }
 
 trk_status trk_set_depth(trk_session* s, const float* depth_m) {
   if (!s || !depth_m) return fail(TRK_ERR_INVALID_ARG, "NULL argument");
   NEED_RESIDENT(s);
-  CK(cudaMemcpyAsync(const_cast<float*>(s->d.depth), depth_m, sizeof(float) * s->d.cam.W * s->d.cam.H,
-                     cudaMemcpyHostToDevice, s->stream));
-  launch_tiles(s->d, s->d.depth, s->stream);
+  TRY(take_depth(s, depth_m));
   return sync_check(s);
 }
 

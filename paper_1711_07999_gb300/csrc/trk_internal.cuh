@@ -6,8 +6,8 @@
 //                v[V] float4, n[V] float4 (w = valid), rec[V] float4 (x,y,z, next-in-bucket bits),
 //                acc[V] Acc4 (sum of p_k - v_i in 2^-30 m, count), vispix[V] int, nbr[V] int4, rg[V] float4
 //   per face   : tris[F] int4 (a,b,c,pad), fn[F] float4 face normals
-//   per pixel  : depth[W*H] float, zbuf[W*H] u64, head[W*H] int, corr[W*H] int, pxy[W*H] float2 (back-projected
-//                points, once per frame), queue[W*H] int, occ (one bit per pixel: its bucket holds a vertex)
+//   per pixel  : zbuf[W*H] u64, head[W*H] int, corr[W*H] int, ppos[W*H] float4 (back-projected points, once per
+//                frame), queue[W*H] int2, occ (one bit per pixel: its bucket holds a vertex)
 //   solver     : partials[nblk][NP*NP] float, A[NP*NP] double, per-candidate theta / DQ tables
 #pragma once
 #include <cstdint>
@@ -285,7 +285,7 @@ size_t vmm_granularity();  // of the current device (0 if the driver's API is un
 cudaError_t vmm_alloc(size_t bytes, VmmBlock* out);
 void vmm_free(VmmBlock* b);
 size_t vmm_bytes_held();   // bytes the library holds through vmm_alloc now, over all devices
-// Copies the frame's depth from src into d.depth (src == d.depth: in place), marks every pixel "no
+// Takes the frame's depth from src: keeps its back-projected points, marks every pixel "no
 // correspondence" and lists the association units (16 x 2 pixels) that hold a valid pixel (the
 // single-session association takes its units from that list).
 void launch_tiles(const Dev& d, const float* src, cudaStream_t st);
@@ -361,8 +361,8 @@ struct Dev {
   float4* pixrec;  // [W*H] first vertex inserted into each pixel's bucket: x, y, z, index bits
   int* head;
   unsigned* occ;   // [H][occ_row(W)] one bit per pixel: its bucket holds a vertex
-  float2* pxy;     // [W*H] pixels with a valid depth: x, y of the back-projected point (session-local frame)
-  int* queue;      // [W*H] pixels whose association search goes on past the thread-owned rings (nearest so far: corr)
+  float4* ppos;    // [W*H] pixels with a valid depth: back-projected point (session-local frame), depth in w
+  int2* queue;     // [W*H] pixels whose association search goes on past the thread-owned rings: (pixel, nearest so far)
   unsigned int* qctl;  // [0] queued pixels, [1] next queue entry to take, [2] association units, [3] unused
   AssocUnit* units;  // [8 ceil(W/16) ceil(H/16)] association units of the frame (up to 32 valid pixels of a tile)
   unsigned long long* zbuf;
@@ -371,7 +371,6 @@ struct Dev {
   int* vispix;
   float4* rg;
   float4* phi0;
-  const float* depth;
   // reductions
   float* partial;   // [nblk_rows][NP*NP]
   int jtj_group;    // 256-vertex blocks per [J r] block (1, 2 or 4)
@@ -387,7 +386,7 @@ struct Dev {
   int precision;          // TRK_PRECISION_*: arithmetic of [J r]^T [J r]
   int shape_solver;       // 0 Jacobi sweeps, 1 coupled PCG
   int association;        // 0 window search, 1 nearest corner of the rasterised triangle
-  const int* adj_off;     // [V + 1] neighbourhood edges of each vertex in both directions (CSR) ...
+  const int* adj_off;     // coupled solve only: [V + 1] neighbourhood edges of each vertex in both directions (CSR) ...
   const int* adj;         // ... sorted by vertex index
   float4 *cg_x, *cg_r, *cg_z, *cg_p, *cg_ap;  // [V] PCG vectors (the direction of odd iterations: in the other phi)
   double* cg;             // [4] rz, alpha, beta, stopped
