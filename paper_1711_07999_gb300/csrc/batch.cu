@@ -46,7 +46,7 @@ struct trk_batch {
   std::vector<unsigned> generations;  // each member's device-state generation when the batch was built
   int device = 0;
   int pose_iters = 0, shape_iters = 0, shape_sweeps = 0, precision = 0, shape_solver = 0;
-  int max_links = 0, max_np = 0;
+  int max_links = 0, max_np = 0, max_window = 0;
   int assoc_blocks = kAssocBlocksPerSM * 152;  // persistent association blocks
   int tail_blocks = kTailBlocksPerSM * 152;  // association-tail blocks (shared by all sessions' queues)
   Dev* d_devs = nullptr;
@@ -102,7 +102,7 @@ void blocks_of(const Dev& d, Kind k, int& gx, int& gy) {
 // One batched frame over a set of sessions: the block tables, the sessions' descriptors and the scratch
 // of the association, wherever they live (a trk_batch's own buffers or a server step's).
 struct FrameView {
-  int B = 0, P = 0, S = 0, sweeps = 0, solver = 0, precision = 0, max_links = 0;
+  int B = 0, P = 0, S = 0, sweeps = 0, solver = 0, precision = 0, max_links = 0, max_window = 0;
   int assoc_blocks = 0, tail_blocks = 0;
   const Dev* d_devs = nullptr;
   Table tables[kKinds];
@@ -133,7 +133,7 @@ void enqueue_frame_view(const FrameView& v, cudaStream_t st) {
     launch_skin_b(grid_of(v, kSkin), v.tables[kSkin].n, L, cur, v.d_ctl, st);
     launch_raster_b(grid_of(v, kTris), v.tables[kTris].n, st);
     launch_visibility_b(grid_of(v, kVerts), v.tables[kVerts].n, st);
-    launch_associate_b(v.d_devs, B, v.d_tiles, v.d_ctl, v.d_prefix, v.assoc_blocks, v.tail_blocks, st);
+    launch_associate_b(v.d_devs, B, v.max_window, v.d_tiles, v.d_ctl, v.d_prefix, v.assoc_blocks, v.tail_blocks, st);
   };
   for (int it = 0; it < P; ++it) {
     geometry();
@@ -169,6 +169,7 @@ FrameView view_of(const trk_batch* b, const std::vector<const Dev*>& host_devs) 
   v.solver = b->shape_solver;
   v.precision = b->precision;
   v.max_links = b->max_links;
+  v.max_window = b->max_window;
   v.assoc_blocks = b->assoc_blocks;
   v.tail_blocks = b->tail_blocks;
   v.d_devs = b->d_devs;
@@ -273,6 +274,7 @@ trk_status batch_create(trk_session* const* sessions, int n_sessions, int assoc_
     const Dev& d = session_dev(s);
     b->max_links = std::max(b->max_links, d.L);
     b->max_np = std::max(b->max_np, d.NP);
+    b->max_window = std::max(b->max_window, d.cam.R);
     b->sessions.push_back(s);
     b->generations.push_back(session_generation(s));
   }
@@ -510,6 +512,7 @@ trk_status batch_step_launch(BatchStep* bs, trk_session* const* ss, int n, const
   v.solver = p0.shape_solver;
   v.precision = p0.precision;
   v.max_links = max_links;
+  for (const Dev* d : hd) v.max_window = std::max(v.max_window, d->cam.R);
   v.assoc_blocks = kAssocBlocksPerSM * 152;
   v.tail_blocks = kTailBlocksPerSM * 152;
   v.d_devs = reinterpret_cast<const Dev*>(dbuf + o_devs);
@@ -615,7 +618,7 @@ trk_status trk_batch_profile(trk_batch* b, const float* const* d_depths, int32_t
     if (!err) err = timed(TRK_STAGE_VISIBILITY, [&] { launch_visibility_b(grid_of(b, kVerts), b->tables[kVerts].n, st); });
     if (!err)
       err = timed(TRK_STAGE_ASSOCIATE, [&] {
-        launch_associate_b(b->d_devs, B, b->d_tiles, b->d_ctl, b->d_prefix, b->assoc_blocks, b->tail_blocks, st);
+        launch_associate_b(b->d_devs, B, b->max_window, b->d_tiles, b->d_ctl, b->d_prefix, b->assoc_blocks, b->tail_blocks, st);
       });
     if (!err)
       err = timed(TRK_STAGE_RESID_JTJ, [&] {
@@ -633,7 +636,7 @@ trk_status trk_batch_profile(trk_batch* b, const float* const* d_depths, int32_t
     launch_skin_b(grid_of(b, kSkin), b->tables[kSkin].n, L, 0, b->d_ctl, st);
     launch_raster_b(grid_of(b, kTris), b->tables[kTris].n, st);
     launch_visibility_b(grid_of(b, kVerts), b->tables[kVerts].n, st);
-    launch_associate_b(b->d_devs, B, b->d_tiles, b->d_ctl, b->d_prefix, b->assoc_blocks, b->tail_blocks, st);
+    launch_associate_b(b->d_devs, B, b->max_window, b->d_tiles, b->d_ctl, b->d_prefix, b->assoc_blocks, b->tail_blocks, st);
     int cur = 0;
     err = timed(TRK_STAGE_SHAPE, [&] {
       cur = launch_shape_b(grid_of(b, kVerts), b->tables[kVerts].n, L, b->shape_sweeps, b->shape_solver, 0, -1, st);

@@ -484,6 +484,7 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
 }
 
 constexpr int kTailWarps = 8;
+constexpr int kMaxRowWindow = 31;     // (the row windows of the occupancy bits hold up to 63 columns)
 constexpr int kTailPerLane = 4;       // buckets a lane loads at once (one session: a warp per pixel)
 constexpr int kBatchTailLanes = 8;    // a batch's tail: lanes per queued pixel ...
 constexpr int kBatchTailPerLane = 4;  // ... and buckets each of them loads at once
@@ -662,8 +663,7 @@ __device__ __forceinline__ void tail_queue(const Dev& d, unsigned n) {
 // four blocks per SM, a frame 1,931 us, from four pixels per warp on 1,983; on two 1,980, from two on 2,086.
 __global__ void __launch_bounds__(32 * kTailWarps, 4) k_associate_tail(Dev d) {
   const unsigned n = *(volatile unsigned*)&d.qctl[0];
-  // (the row windows of the occupancy bits hold up to 63 columns)
-  if (n > 2 * gridDim.x / 152 * gridDim.x * kTailWarps && d.cam.R <= 31) tail_queue<kBatchTailLanes, kBatchTailPerLane, true>(d, n);
+  if (n > 2 * gridDim.x / 152 * gridDim.x * kTailWarps && d.cam.R <= kMaxRowWindow) tail_queue<kBatchTailLanes, kBatchTailPerLane, true>(d, n);
   else tail_queue<32, kTailPerLane, false>(d, n);
 }
 
@@ -699,6 +699,7 @@ __global__ void __launch_bounds__(1024) k_tail_prefix(const Dev* devs, int n_ses
 // A batch: the lane groups take entries of the concatenated queues of all sessions, group g the g-th, then
 // the rest from one counter; an entry's session is found in the prefix and its descriptor read through
 // the cache.
+template <bool kRows>
 __global__ void __launch_bounds__(32 * kTailWarps, kTailBlocksPerSM) k_associate_tail_batch(const Dev* devs, int n_sessions,
                                                                           const unsigned* global_prefix, unsigned* ctl) {
   constexpr int GL = kBatchTailLanes;
@@ -734,10 +735,7 @@ __global__ void __launch_bounds__(32 * kTailWarps, kTailBlocksPerSM) k_associate
       if (prefix[mid] <= item) lo = mid; else hi = mid - 1;
     }
     const Dev& d = devs[lo];
-    // (the row windows of the occupancy bits hold up to 63 columns)
-    const bool got = d.cam.R <= 31 ? tail_item<GL, kBatchTailPerLane, true>(d, item - prefix[lo], gl, gmask)
-                                   : tail_item<GL, kBatchTailPerLane, false>(d, item - prefix[lo], gl, gmask);
-    if (got && gl == 0) atomicAdd(&d.stats[0], 1);
+    if (tail_item<GL, kBatchTailPerLane, kRows>(d, item - prefix[lo], gl, gmask) && gl == 0) atomicAdd(&d.stats[0], 1);
     if (groups >= total) break;
     unsigned next = 0;
     if (gl == 0) next = groups + atomicAdd(&ctl[2], 1u);
@@ -819,11 +817,15 @@ void launch_raster_b(const BatchGrid& g, int nblk, cudaStream_t st) {
 void launch_visibility_b(const BatchGrid& g, int nblk, cudaStream_t st) {
   if (nblk > 0) k_visibility_b<<<nblk, kBlock, 0, st>>>(g);
 }
-void launch_associate_b(const Dev* devs, int n_sessions, const AssocUnit* tiles, unsigned* ctl, unsigned* prefix,
-                        int assoc_blocks, int tail_blocks, cudaStream_t st) {
+void launch_associate_b(const Dev* devs, int n_sessions, int max_window, const AssocUnit* tiles, unsigned* ctl,
+                        unsigned* prefix, int assoc_blocks, int tail_blocks, cudaStream_t st) {
   k_associate<<<assoc_blocks, kBlock, 0, st>>>(devs, tiles, ctl, Dev{});
   if (n_sessions > kInBlockPrefix) k_tail_prefix<<<1, 1024, 0, st>>>(devs, n_sessions, prefix);
-  k_associate_tail_batch<<<tail_blocks, 32 * kTailWarps, 0, st>>>(devs, n_sessions, prefix, ctl);
+  // (one kernel for both searches would spill registers: they together are within one session's launch bounds only)
+  if (max_window <= kMaxRowWindow)
+    k_associate_tail_batch<true><<<tail_blocks, 32 * kTailWarps, 0, st>>>(devs, n_sessions, prefix, ctl);
+  else
+    k_associate_tail_batch<false><<<tail_blocks, 32 * kTailWarps, 0, st>>>(devs, n_sessions, prefix, ctl);
 }
 
 // Back-projects each session's depth frame at srcs[session] into the session's points, one 16 x 16

@@ -414,8 +414,9 @@ struct BatchGrid;
 void launch_skin_b(const BatchGrid& g, int nblk, int max_links, int phi_buf, unsigned* ctl, cudaStream_t st);
 void launch_raster_b(const BatchGrid& g, int nblk, cudaStream_t st);
 void launch_visibility_b(const BatchGrid& g, int nblk, cudaStream_t st);
-void launch_associate_b(const Dev* devs, int n_sessions, const AssocUnit* units, unsigned* ctl, unsigned* prefix,
-                        int assoc_blocks, int tail_blocks, cudaStream_t st);
+// max_window: the largest window half-size of the sessions
+void launch_associate_b(const Dev* devs, int n_sessions, int max_window, const AssocUnit* units, unsigned* ctl,
+                        unsigned* prefix, int assoc_blocks, int tail_blocks, cudaStream_t st);
 void launch_gather_depth_b(const BatchGrid& g, int nblk, const float* const* srcs, AssocUnit* units, unsigned* ctl,
                            cudaStream_t st);
 // fork (may be null): streams on which the [J r] launches of the tile width classes run beside each other.
