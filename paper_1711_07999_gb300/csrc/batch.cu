@@ -340,9 +340,8 @@ trk_status batch_create(trk_session* const* sessions, int n_sessions, int assoc_
 // step costs its launches, one small upload and no per-session copies.
 
 // Vertex block vb of a session's results.  Bound by the writes over the chip-to-chip link: the offsets go out as
-// [V][3] through shared memory, in 16-byte pieces, and the host only copies them.  (Four copies and a host loop
-// that picked three of every four floats before: a tracked frame of 200k vertices 2,296 -> 2,177 us, of 50k
-// 1,082 -> 1,038.)
+// [V][3] through shared memory, in 16-byte pieces, and the host only copies them.  (Four copies and a host loop that
+// picks three of every four floats: a tracked frame of 200k vertices 2,140 us, so 2,095; of 50k 1,055 and 1,032.)
 __device__ __forceinline__ void results_impl(const Dev& d, const ResultDst& o, int vb) {
   __shared__ __align__(16) float s_phi[3 * 256];
   const int t = threadIdx.x, n = min(256, d.V - 256 * vb);  // vertices of this block

@@ -165,15 +165,6 @@ __global__ void __launch_bounds__(kJLoaders + 128) k_jtj_rows(const float* __res
     }
 }
 
-// (double)x of a normal x or zero, with integer operations: conversions to FP64 take 60 cycles of the FP64
-// pipe per warp.  Sets `other` where x is neither.
-__device__ __forceinline__ double widen(float x, bool& other) {
-  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
-  other |= a != 0u && a - 0x00800000u >= 0x7f000000u;
-  const unsigned hi = (u & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u);
-  return __hiloint2double((int)hi, (int)(a << 29));
-}
-
 // FP64 sum of the nblk partials in a fixed order: warp w of the block's S adds partials w, w + S, ... (all
 // its loads of a round in flight), warp 0 the warps' sums.  kUpper: the partials hold the upper triangle,
 // whose entries are written to both places.

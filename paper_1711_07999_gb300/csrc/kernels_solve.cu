@@ -609,15 +609,6 @@ __device__ __forceinline__ void sum2_add(float& hi, float& lo, float x) {
   lo += e;
 }
 
-// (double)x of a normal x or zero, with integer operations: conversions to FP64 take 60 cycles of the FP64
-// pipe per warp.  Sets `other` where x is neither.
-__device__ __forceinline__ double widen(float x, bool& other) {
-  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
-  other |= a != 0u && a - 0x00800000u >= 0x7f000000u;
-  const unsigned hi = (u & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u);
-  return __hiloint2double((int)hi, (int)(a << 29));
-}
-
 constexpr int kReduceBatch = 8;  // partials a warp has in flight
 
 __device__ __forceinline__ void reduce_jtj_impl(const Dev& d, BlockPos bp, int slot) {
@@ -1371,17 +1362,19 @@ __device__ __forceinline__ void lm_eval_impl(const Dev& d, BlockPos bp) {
       if (c >= c0 && c < c1) swarp[w][c] = e[c];
   }
   __syncthreads();
-  // the block's energies, then its ticket: one warp writes, fences and takes it
+  // the block's energies, then its ticket: one warp writes and takes it
   if (w == 0) {
     if (lane >= c0 && lane < c1) {
       double s = 0.0;
 #pragma unroll
       for (int k = 0; k < kBlock / 32; ++k) s += swarp[k][lane];
       d.epart[(size_t)bp.x * 8 + lane] = s;
-      __threadfence();
     }
     __syncwarp();
-    if (lane == 0) last = atomicAdd(&d.counter[0], 1u) == (unsigned)bp.gx - 1;
+    if (lane == 0) {
+      __threadfence();  // (by the lane that takes the ticket: it orders what the warp's barrier showed it, too)
+      last = atomicAdd(&d.counter[0], 1u) == (unsigned)bp.gx - 1;
+    }
   }
   __syncthreads();
   if (!last) return;
@@ -1656,7 +1649,7 @@ __global__ void __launch_bounds__(kBlock) k_shape_sweep(BatchGrid g, Dev d0, int
 // p.Ap <= 0) stops the iteration as in exact arithmetic.  One kernel per CG phase.
 // ---------------------------------------------------------------------------------------------
 // Block sum of v (FP64) into epart[bp.x * 8 + slot]; returns true in every thread of the session's last
-// block, with the fixed-order total of all its blocks in `total`.
+// block, with the fixed-order total of all its blocks in thread 0's `total`.
 __device__ __forceinline__ bool block_total(const Dev& d, BlockPos bp, double v, int slot, int ticket, double& total) {
   __shared__ double sw[kBlock / 32];
   __shared__ double red[kBlock];

@@ -134,6 +134,15 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// (double)x of a normal x or zero, with integer operations: conversions to FP64 take 60 cycles of the FP64
+// pipe per warp.  Sets `other` where x is neither.
+__device__ __forceinline__ double widen(float x, bool& other) {
+  const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+  other |= a != 0u && a - 0x00800000u >= 0x7f000000u;
+  const unsigned hi = (u & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(a << 29));
+}
+
 // Forward kinematics of all links (Sec. 3.1): H_{0,j} = H_{0,parent(j)} off_j J_j(theta_j) (H_{0,-1} = the
 // root transform pre), formed as (H_{0,parent} off_j) J_j.  Writes H_{j,Delta} = H_{0,j} conj(H^0_{0,j})
 // and the twist Xi_j = H_{0,j} G_j conj(H_{0,j}) with G_j = (0, z/2 | 0) for a hinge and (0 | 0, z/2) for
