@@ -236,7 +236,7 @@ void launch_visibility(const Dev& d, cudaStream_t st) {
 // k_associate: rings 0..kRingsPerThread by the pixel's own thread or by four lanes (see there).  Pixels still open
 // after that (the bound of ring 1 is ~4 mm at 2-3 m: pixels whose nearest vertex is farther, in the first iterations
 // of a frame, at silhouettes and where vertices are sparse) go to a queue that the tail kernels drain with a group of
-// lanes per pixel (a warp for one session, kBatchTailLanes lanes in a batch), the lanes splitting the next rings'
+// lanes per pixel (a warp for one session's short queue, else kBatchTailLanes lanes), the lanes splitting the next rings'
 // buckets and combining (d^2, index) keys with a group min.
 // The pixel's offset p - v_i is added to the vertex's fixed-point sums (integer atomics: the sums do
 // not depend on the order of the additions).
@@ -485,8 +485,8 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
 
 constexpr int kTailWarps = 8;
 constexpr int kMaxRowWindow = 31;     // (the row windows of the occupancy bits hold up to 63 columns)
-constexpr int kTailPerLane = 4;       // buckets a lane loads at once (one session: a warp per pixel)
-constexpr int kBatchTailLanes = 8;    // a batch's tail: lanes per queued pixel ...
+constexpr int kTailPerLane = 4;       // buckets a lane loads at once (one session's short queue: a warp per pixel)
+constexpr int kBatchTailLanes = 8;    // a batch's tail and a long queue: lanes per queued pixel ...
 constexpr int kBatchTailPerLane = 4;  // ... and buckets each of them loads at once
 
 // The rings beyond the thread-owned ones for queue entry `item` of session d, by a group of GL lanes (lanes
@@ -494,10 +494,10 @@ constexpr int kBatchTailPerLane = 4;  // ... and buckets each of them loads at o
 // ring's 8r buckets (up to kTailPerLane each per round trip, heads and first records loaded together) and
 // combine (d^2, index) keys with a group min.  Returns, in every lane of the group, whether the pixel got a
 // correspondence (its first lane writes it and adds the pixel's sums).
-// One session's tail takes a warp per pixel (its queue is short and its latency is the slowest pixel's
-// rings); a batch's takes 8 lanes per pixel (four pixels per warp: throughput over many queues).
+// One session's tail takes a warp per pixel while its queue is short (its latency is then the slowest pixel's
+// rings); a long queue and a batch's take 8 lanes per pixel (four pixels per warp: throughput).
 //
-// A batch's lanes (kRows) take a row of the square each instead and read which of its buckets hold a vertex from
+// Those lanes (kRows) take a row of the square each instead and read which of its buckets hold a vertex from
 // the occupancy bits, three words for the rings of a round together, so that an empty bucket -- most of
 // them at silhouettes and where the mesh is coarser than the image -- costs no load; a round takes rings
 // r0 .. r0 + 1 first, four more rings after that.
