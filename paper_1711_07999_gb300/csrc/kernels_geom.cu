@@ -485,13 +485,12 @@ __device__ __forceinline__ void associate4_impl(const Dev& d, int px, int py, bo
 
 constexpr int kTailWarps = 8;
 constexpr int kMaxRowWindow = 31;     // (the row windows of the occupancy bits hold up to 63 columns)
-constexpr int kTailPerLane = 4;       // buckets a lane loads at once (one session's short queue: a warp per pixel)
 constexpr int kBatchTailLanes = 8;    // a batch's tail and a long queue: lanes per queued pixel ...
 constexpr int kBatchTailPerLane = 4;  // ... and buckets each of them loads at once
 
 // The rings beyond the thread-owned ones for queue entry `item` of session d, by a group of GL lanes (lanes
 // gl = lane % GL of the group starting at lane gbase, gmask naming them): the lanes split each
-// ring's 8r buckets (up to kTailPerLane each per round trip, heads and first records loaded together) and
+// ring's 8r buckets (up to PL each per round trip, heads and first records loaded together) and
 // combine (d^2, index) keys with a group min.  Returns, in every lane of the group, whether the pixel got a
 // correspondence (its first lane writes it and adds the pixel's sums).
 // One session's tail takes a warp per pixel while its queue is short (its latency is then the slowest pixel's
@@ -661,10 +660,14 @@ __device__ __forceinline__ void tail_queue(const Dev& d, unsigned n) {
 // throughput and goes eight lanes to a pixel, as a batch's does (640x480 with every pixel valid: 402 -> 153 us the
 // association).  Below that it loses where the mesh is finer than the image: 200k vertices at 1280x720 on
 // four blocks per SM, a frame 1,931 us, from four pixels per warp on 1,983; on two 1,980, from two on 2,086.
+// kPerLane: buckets a lane loads at once in the former (launch_associate).
+template <int kPerLane>
 __global__ void __launch_bounds__(32 * kTailWarps, 4) k_associate_tail(Dev d) {
   const unsigned n = *(volatile unsigned*)&d.qctl[0];
-  if (n > 2 * gridDim.x / 152 * gridDim.x * kTailWarps && d.cam.R <= kMaxRowWindow) tail_queue<kBatchTailLanes, kBatchTailPerLane, true>(d, n);
-  else tail_queue<32, kTailPerLane, false>(d, n);
+  if (n > 2 * gridDim.x / 152 * gridDim.x * kTailWarps && d.cam.R <= kMaxRowWindow)
+    tail_queue<kBatchTailLanes, kBatchTailPerLane, true>(d, n);
+  else
+    tail_queue<32, kPerLane, false>(d, n);
 }
 
 constexpr int kInBlockPrefix = 32 * kTailWarps;  // sessions whose prefix the tail's blocks form themselves
@@ -748,12 +751,13 @@ void launch_associate(const Dev& d, cudaStream_t st) {
   k_associate<<<min((nunits + kBlock / 32 - 1) / (kBlock / 32), kAssocBlocksPerSM * 152), kBlock, 0, st>>>(nullptr, nullptr,
                                                                                                    nullptr, d);
   // Blocks of the tail: most sessions track beside others, whose work the blocks of a short queue hold up (32 sessions on
-  // their own streams, frames/s at two and four blocks per SM: 5k vertices at 160x120 27,400 and 23,300, 50k at
-  // 640x480 5,050 and 4,885; one session alone: 50k 955 and 947 us a frame).  A larger image queues more pixels
-  // than two have warps for (200k vertices at 1280x720: 1,957 and 1,863 us a frame, eight sessions 1,313 and
-  // 1,272 frames/s).
-  const int per_sm = d.cam.W * d.cam.H > 640 * 480 ? 4 : 2;
-  k_associate_tail<<<per_sm * 152, 32 * kTailWarps, 0, st>>>(d);
+  // their own streams, frames/s at two and four blocks per SM: 5k vertices at 160x120 27,300 and 23,400, 50k at
+  // 640x480 5,170 and 5,015; one session of 50k alone 943 and 935 us a frame).  A larger image queues more
+  // pixels than two have warps for (200k vertices at 1280x720: 1,957 and 1,863 us a frame, eight sessions
+  // 1,313 and 1,272 frames/s).  Two buckets per lane hold rings 2 and 3, where most searches of a small image end;
+  // four hold rings 2 to 5 (a frame of 5k, 50k and 200k vertices: two 654, 943 and 1,882 us, four 662, 948 and 1,857).
+  if (d.cam.W * d.cam.H > 640 * 480) k_associate_tail<4><<<4 * 152, 32 * kTailWarps, 0, st>>>(d);
+  else k_associate_tail<2><<<2 * 152, 32 * kTailWarps, 0, st>>>(d);
 }
 
 // Appends this block's tile's association units to list: its pixels with a valid depth, in row-major
